@@ -64,8 +64,6 @@ NCU_TRAFFIC = {
     "fem_bwd_elem_kernel<3,LAPLACE_P1,JAC_SAVED>": {"bytes_per_launch": 1321.0e6, "src": "4a6c95b7dc30da51"},
     "fem_fwd_kernel<3,LAPLACE_P1,JAC_COMP>": {"bytes_per_launch": 962.3e6, "src": "7c0682f050b938ea"},
     "vertex_reduce_kernel<3>": {"bytes_per_launch": 149.3e6, "src": "2fda9ba9be91ca76"},
-    # tile pass + entry pass of one call, 96^3 capture scaled by the elements (records grow alike)
-    "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 2232.3e6, "src": "2fcf5baed442a38c"},
 }
 
 
@@ -936,10 +934,8 @@ def run_assemble(args):
             continue
         err = max(err, max(abs(got.get(k, 0.0) - ref[k]) for k in ref) / bound[v])
     nnz, R2 = asm.nnz, asm.n_records
-    T = (E + 31) // 32
-    # tile pass: A, run words, record cells, tile offsets/runs, record slots read, records written;
-    # entry pass: entry offsets, records read (contiguous), values written
-    byts = E * 64 + E * 4 + R2 * 2 + T * 6 + R2 * 4 + (nnz + 1) * 4 + R2 * 4 + R2 * 4 + nnz * 4
+    # A, an 8-byte slot per incidence, row offsets read; values written
+    byts = E * 64 + E * 4 * 8 + (V + 1) * 4 + nnz * 4
     peak, peak_kind = hbm_peak()
     gbs = byts / (asm_ms * 1e-3) / 1e9
     out = {"metric": METRIC, "value": E / (asm_ms * 1e-3), "unit": "elements/s", "n_gpus": 1,
@@ -950,7 +946,7 @@ def run_assemble(args):
                                   f"{R2:,} tile records), "
                                   "deterministic (per 32-element tile in element order, then in tile order)",
                       "elements": E, "nnz": nnz, "l2": f"no flush: {byts / 1e9:.1f} GB moved per step"},
-           "roofline": {"bound": "hbm", "kernel": "fem_assemble<LAPLACE_P1> (tile pass + entry pass, one call)",
+           "roofline": {"bound": "hbm", "kernel": "fem_assemble<LAPLACE_P1> (assemble_blocks_kernel, one call)",
                         "achieved": gbs, "peak": peak,
                         "unit": "GB/s", "frac": gbs / peak, "peak_kind": f"{peak_kind} copy bandwidth",
                         "traffic": ncu_traffic("fem_assemble<LAPLACE_P1>"), "algorithmic_bytes": byts},
@@ -960,7 +956,7 @@ def run_assemble(args):
            "timing": {"repeats": ra["repeats"], "ms_per_step_min": ra["ms_min"], "ms_per_step_max": ra["ms_max"],
                       "statistic": "median over repeats of K-step timed regions"},
            "clocks": ra["clocks"], "forward_clocks": rf["clocks"],
-           "gpu_launches": 2 * args.steps}  # tile pass + entry pass per call
+           "gpu_launches": args.steps}  # one kernel per call
     # the P2 Laplacian over its vertex and edge unknowns (row kernel, element order)
     del A, vals
     torch.cuda.synchronize()

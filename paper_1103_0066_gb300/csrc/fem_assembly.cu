@@ -13,27 +13,20 @@
 //                distinct ones (the row's columns, increasing), and stores for
 //                every incidence t and local vertex j the position of
 //                conn[e][j] among them (colpos, one byte)
-// Scalar forms, tile records (built once per connectivity, after the pattern):
-//   per 32-element tile (one warp): the tile's distinct vertices ("runs", R_t
-//   of them) and every slot's run index (one byte); the distinct (row run,
-//   column run) cells the tile touches, each one RECORD (records numbered in
-//   tile order), the entry -> records CSR (eoff, rec_list) and its inverse,
-//   every record's slot in entry order (rec_dest) -- the tile / record scheme
-//   of the adjoint's reduction, keyed by matrix entry.
-// Assembly of the scalar forms (fem_assemble):
-//   1. one warp per tile reads its element matrices coalesced into shared
-//      memory and adds them, element by element, into a dense R_t x R_t tile
-//      matrix (an element's cells are distinct, so a step has no conflicts);
-//      each cell is the sum of its contributions in element order.  Each cell
-//      is written as a record to its slot in entry order (tiles with R_t above
-//      kTileRuns take an exact per-record scan of the tile instead);
-//   2. one thread per entry sums its records, which lie side by side in tile
-//      order, so the pass reads them contiguously.
+//   row blocks : (P1 forms and elasticity) the incidences of 32 / B^2
+//                consecutive rows, padded to the longest row of the block and
+//                interleaved, so that the lanes of a warp read them coalesced
+// Assembly (fem_assemble), P1 forms and elasticity: one kernel, a warp per row
+// block, a lane per row and block component.  A lane walks its row's
+// incidences in element order, reads the element row's NV entries of its
+// component (16 bytes on tets) and adds them to its own column sums in shared
+// memory.  No two lanes share a sum, so the order of every sum is the lane's
+// program order:
+//   scalar P1 forms: per 32-element tile the contributions in element order,
+//                    then those tile sums in tile order (the build marks the
+//                    first and the last contribution of every (tile, entry));
+//   elasticity     : all contributions in element order.
 // Every entry is therefore a fixed-order sum, bitwise reproducible.
-// P1 elasticity (d x d blocks) takes the row kernel: one thread per row walks
-// its incidences in increasing element order and adds the element's rows into
-// the row's columns, accumulating in shared memory (rows of up to kFastCols
-// columns) or in place in the output.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -48,22 +41,15 @@ namespace {
 
 constexpr int kRowCap = 512;    // candidate columns per row (incidences x (d+1))
 constexpr int kMaxCols = 255;   // distinct columns per row (one-byte positions)
-constexpr int kFastCols = 32;   // rows accumulated in shared memory
+constexpr int kFastCols = 32;   // columns of a row accumulated in shared memory
 constexpr int kPatWarps = 4;
-constexpr int kAsmThreads = 64;
-constexpr int kTileRuns = 36;  // dense tile matrix side (distinct vertices of a 32-element tile)
-// Row stride of a tile's cells, cell = row run * stride + column run: at least
-// kCellStride, so that the 16 cells of an element (4 runs x 4 runs) spread over
-// the shared-memory banks (a stride of the run count itself, near 32 on a
-// cell-major mesh, puts them in a few banks); the run count when it is larger.
-// Cells ordered by value are in (row run, column run) order either way.
-constexpr int kCellStride = 34;
-__host__ __device__ __forceinline__ int cell_stride(int nr) { return nr > kCellStride ? nr : kCellStride; }
-constexpr int kTileWarps = 1;  // warps per CTA of the tile pass (no CTA-wide barrier: finest sharing of shared memory)
-constexpr int kTileCap = 128;  // slots of a 32-element tile (tets: 4 per element)
-constexpr int kCellCap = 512;  // contributions of a 32-element tile (tets: 16 per element)
-constexpr int kDestRegs = 8;   // record slots a lane of the tile pass holds in registers (tiles of up to 256 records)
-constexpr int kHalvesDisjoint = 0x100;  // tile_runs flag: elements 0-15 and 16-31 share no cell
+
+// Lanes a row takes (one per component of its blocks) and rows of a row block.
+__host__ __device__ constexpr int row_lanes(int B) { return B * B; }
+__host__ __device__ constexpr int block_rows(int B) { return 32 / (B * B); }
+// Marks in a byte of a slot's column word (scalar forms): the contribution is
+// the first / the last one of its 32-element tile to its entry.
+constexpr uint32_t kFirst = 0x40, kLast = 0x80;
 
 enum : int { ASM_ROW_TOO_LONG = 1, ASM_BAD_VERTEX = 2, ASM_REPEATED_VERTEX = 4 };
 
@@ -172,437 +158,326 @@ __global__ void __launch_bounds__(kPatWarps * 32)
   }
 }
 
-// N = rows of A_e = NV * B; local unknown (c, i) is row c * NV + i.
-// Incidences are taken in groups of kAsmBatch: all their loads (incidence,
-// column positions, element rows) are issued before the group's additions,
-// which then run in increasing incidence order.  For tets the four column
-// positions are one 4-byte load and an element row of a scalar form is one
-// 16-byte load.
-constexpr int kAsmBatch = 4;
+// ------------------------------------------------------------------ row blocks (P1 forms and elasticity)
 
+// Steps of each row block: its longest row's incidences; 0 where the kernel
+// has to scan instead, because a row has more than kFastCols columns or an
+// element of it lists the row's vertices twice (its positions then coincide).
 template <int NV, int B>
-__global__ void __launch_bounds__(kAsmThreads)
-    assemble_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
-                    const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                    const float* __restrict__ A, int64_t n_vert, float* __restrict__ val, int vec_A,
-                    const int32_t* __restrict__ n_rows_dev) {
-  constexpr int N = NV * B, BB = B * B;
-  extern __shared__ float acc_s[];  // [kAsmThreads][kFastCols * BB + 1]
-  float* acc = acc_s + threadIdx.x * (kFastCols * BB + 1);
-  if (n_rows_dev) n_vert = *n_rows_dev;  // rows known only on the device (P2 unknowns)
-  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n_vert;
-       v += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t rp = row_ptr[v];
-    const int len = row_ptr[v + 1] - rp;
-    const bool fast = len <= kFastCols;
-    float* dst = fast ? acc : val + int64_t(rp) * BB;
-    for (int q = 0; q < len * BB; ++q) dst[q] = 0.f;
-    const int32_t t1 = inc_off[v + 1];
-    for (int32_t t0 = inc_off[v]; t0 < t1; t0 += kAsmBatch) {
-      int32_t s[kAsmBatch];
-      uint8_t pos[kAsmBatch][NV];
-      float a[kAsmBatch][B][B][NV];
+__global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ row_ptr,
+                                   const uint8_t* __restrict__ colpos, int64_t n_vert, int32_t* steps) {
+  constexpr int G = block_rows(B);
+  const int64_t nblk = (n_vert + G - 1) / G;
+  for (int64_t b = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; b < nblk; b += int64_t(gridDim.x) * blockDim.x) {
+    int n = 0;
+    bool fast = true;
+    for (int64_t v = b * G; v < (b + 1) * G && v < n_vert; ++v) {
+      fast &= row_ptr[v + 1] - row_ptr[v] <= kFastCols;
+      const int c = inc_off[v + 1] - inc_off[v];
+      n = c > n ? c : n;
+      if constexpr (B > 1)  // the scalar forms refuse such elements
+        for (int32_t t = inc_off[v]; fast && t < inc_off[v + 1]; ++t)
 #pragma unroll
-      for (int u = 0; u < kAsmBatch; ++u) s[u] = t0 + u < t1 ? __ldg(inc + t0 + u) : 0;
+          for (int i = 0; i < NV; ++i)
 #pragma unroll
-      for (int u = 0; u < kAsmBatch; ++u) {
-        const int32_t t = t0 + u < t1 ? t0 + u : t0;
-        if constexpr (NV == 4) {
-          const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(colpos) + t);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) pos[u][j] = uint8_t(w >> (8 * j));
-        } else {
-#pragma unroll
-          for (int j = 0; j < NV; ++j) pos[u][j] = __ldg(colpos + int64_t(t) * NV + j);
-        }
-        const int i = s[u] % NV;
-        const float* Ae = A + int64_t(s[u] / NV) * (N * N);
-#pragma unroll
-        for (int c = 0; c < B; ++c)
-#pragma unroll
-          for (int c2 = 0; c2 < B; ++c2) {
-            const float* src = Ae + (c * NV + i) * N + c2 * NV;
-            if constexpr (NV == 4) {
-              if (vec_A) {  // 16-byte aligned: (c*NV + i)*N + c2*NV is a multiple of 4
-                const float4 q = __ldg(reinterpret_cast<const float4*>(src));
-                a[u][c][c2][0] = q.x;
-                a[u][c][c2][1] = q.y;
-                a[u][c][c2][2] = q.z;
-                a[u][c][c2][3] = q.w;
-                continue;
-              }
-            }
-#pragma unroll
-            for (int j = 0; j < NV; ++j) a[u][c][c2][j] = __ldg(src + j);
-          }
-      }
-#pragma unroll
-      for (int u = 0; u < kAsmBatch; ++u) {
-        if (t0 + u >= t1) break;
-#pragma unroll
-        for (int c = 0; c < B; ++c)
-#pragma unroll
-          for (int j = 0; j < NV; ++j)
-#pragma unroll
-            for (int c2 = 0; c2 < B; ++c2) dst[pos[u][j] * BB + c * B + c2] += a[u][c][c2][j];
-      }
+            for (int j = i + 1; j < NV; ++j) fast &= colpos[int64_t(t) * NV + i] != colpos[int64_t(t) * NV + j];
     }
-    if (fast) {
-      float* out = val + int64_t(rp) * BB;
-      for (int q = 0; q < len * BB; ++q) out[q] = acc[q];
-    }
+    steps[b] = fast ? n : 0;
   }
 }
 
-// ------------------------------------------------------------------ tile records (scalar forms)
-
-// Sorts n_pow2 keys in shared memory (bitonic, one warp).
-template <class K>
-__device__ __forceinline__ void warp_bitonic(K* key, int P, int lane) {
-  for (int k2 = 2; k2 <= P; k2 <<= 1)
-    for (int jj = k2 >> 1; jj > 0; jj >>= 1) {
-      for (int i = lane; i < P; i += 32) {
-        const int ixj = i ^ jj;
-        if (ixj > i) {
-          const bool up = (i & k2) == 0;
-          const K x = key[i], y = key[ixj];
-          if ((x > y) == up) {
-            key[i] = y;
-            key[ixj] = x;
-          }
-        }
-      }
-      __syncwarp();
-    }
-}
-
-// One warp per 32-element tile.  PASS 1 counts the tile's cells (records);
-// PASS 2 writes the slot run indices, R_t, each record's cell (r_v * R_t + r_w)
-// and its matrix entry (CSR position of (v, w)).
-template <int NV, bool WRITE>
-__global__ void __launch_bounds__(kPatWarps * 32)
-    tile_cells_kernel(const int32_t* __restrict__ conn, int64_t n_elem, const int32_t* __restrict__ row_ptr,
-                      const int32_t* __restrict__ col_idx, int32_t* tile_nrec, const int32_t* __restrict__ tile_rec,
-                      uint32_t* run_word, uint16_t* tile_runs, uint16_t* rec_cell, int32_t* rec_entry, int32_t* flag) {
-  __shared__ uint64_t skey_s[kPatWarps][kTileCap];
-  __shared__ uint32_t ckey_s[kPatWarps][kCellCap];
-  __shared__ int32_t runv_s[kPatWarps][kTileCap];
-  __shared__ uint8_t runi_s[kPatWarps][kTileCap];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint64_t* skey = skey_s[warp];
-  uint32_t* ckey = ckey_s[warp];
-  int32_t* runv = runv_s[warp];
-  uint8_t* runi = runi_s[warp];
-  constexpr int NS = 32 * NV;                  // slots of a full tile
-  constexpr int PS = NS <= 64 ? 64 : 128;      // power of two >= NS (and >= 32)
-  constexpr int NC = 32 * NV * NV;             // contributions of a full tile
-  constexpr int PC = NC <= 256 ? 256 : 512;
-  const int64_t ntiles = (n_elem + 31) / 32;
-  const int64_t stride = int64_t(gridDim.x) * kPatWarps;
-  for (int64_t t = int64_t(blockIdx.x) * kPatWarps + warp; t < ntiles; t += stride) {
-    const int64_t e0 = t * 32;
-    const int ne = int(n_elem - e0 < 32 ? n_elem - e0 : 32);
-    const int ns = ne * NV;
-    // 1. slots sorted by (vertex, slot): runs and run index per slot
-    for (int i = lane; i < PS; i += 32) {
-      uint64_t k = ~0ull;
-      if (i < ns) k = (uint64_t(uint32_t(conn[e0 * NV + i])) << 16) | uint64_t(i);
-      skey[i] = k;
-    }
-    __syncwarp();
-    warp_bitonic(skey, PS, lane);
-    int nr = 0;
-    for (int r = 0; r < ns; r += 32) {
-      const int i = r + lane;
-      const bool head = i < ns && (i == 0 || (skey[i] >> 16) != (skey[i - 1] >> 16));
-      const uint32_t bal = __ballot_sync(0xffffffffu, head);
-      const uint32_t upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);  // lanes <= this one
-      const int run = nr + __popc(bal & upto) - 1;  // heads up to this position, minus one
-      if (head) runv[run] = int32_t(skey[i] >> 16);
-      if (i < ns) runi[int(skey[i] & 0xFFFF)] = uint8_t(run);
-      nr += __popc(bal);
-    }
-    __syncwarp();
-    // 2. cells of the tile's contributions, in (row run, column run) order; the
-    //    key keeps the element (low 6 bits) to tell whether the two half-tiles
-    //    (elements 0-15, 16-31) share a cell
-    const int ncell = ne * NV * NV;
-    int rep = 0;
-    for (int c = lane; c < PC; c += 32) {
-      uint32_t k = 0xFFFFFFFFu;
-      if (c < ncell) {
-        const int el = c / (NV * NV), ij = c % (NV * NV), i = ij / NV, j = ij % NV;
-        const int ri = runi[el * NV + i], rj = runi[el * NV + j];
-        if (i != j && ri == rj) rep = 1;  // an element repeats a vertex
-        k = (uint32_t(ri * cell_stride(nr) + rj) << 6) | uint32_t(el);
-      }
-      ckey[c] = k;
-    }
-    if (__any_sync(0xffffffffu, rep) && lane == 0) atomicOr(flag, ASM_REPEATED_VERTEX);
-    __syncwarp();
-    warp_bitonic(ckey, PC, lane);
-    int nu = 0, shared = 0;
-    for (int r = 0; r < ncell; r += 32) {
-      const int i = r + lane;
-      const bool head = i < ncell && (i == 0 || (ckey[i] >> 6) != (ckey[i - 1] >> 6));
-      // within a cell the elements ascend: the halves meet where a lower-half
-      // element is followed by an upper-half one
-      if (i + 1 < ncell && (ckey[i] >> 6) == (ckey[i + 1] >> 6) && (ckey[i] & 63u) < 16u && (ckey[i + 1] & 63u) >= 16u)
-        shared = 1;
-      const uint32_t bal = __ballot_sync(0xffffffffu, head);
-      if constexpr (WRITE) {
-        if (head) {
-          const int32_t rec = tile_rec[t] + nu + __popc(bal & ((1u << lane) - 1u));
-          const uint32_t cell = ckey[i] >> 6;
-          const int32_t v = runv[cell / cell_stride(nr)], w = runv[cell % cell_stride(nr)];
-          int lo = row_ptr[v], hi = row_ptr[v + 1];  // position of w in row v
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (col_idx[mid] < w)
-              lo = mid + 1;
-            else
-              hi = mid;
-          }
-          rec_cell[t * kCellCap + (rec - tile_rec[t])] = uint16_t(cell);  // the tile's 512-entry slot
-          rec_entry[rec] = lo;
-        }
-      }
-      nu += __popc(bal);
-    }
-    shared = __any_sync(0xffffffffu, shared);
-    if constexpr (!WRITE) {
-      if (lane == 0) tile_nrec[t] = nu;
-    } else {
-      uint32_t wd = 0;
-      if (lane < ne) {
+// The slots of every row: (element slot e * NV + i, one byte per local vertex
+// j: the column position, for the scalar forms with the tile marks), padded
+// with element slot -1 to the block's steps.  A tile's incidences of one row
+// are neighbours (the list is in element order), so the marks come from a look
+// at them.  first marks are counted: one per (tile, entry), the tile records.
+template <int NV, int B>
+__global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ blk_off,
+                                  int64_t n_vert, int64_t slot_cap, int2* __restrict__ slots, int32_t* n_records) {
+  constexpr int G = block_rows(B);
+  const int64_t nblk = (n_vert + G - 1) / G;
+  const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
+  int nrec = 0;
+  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n_vert; v += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t b = v / G;
+    const int32_t s0 = blk_off[b], steps = blk_off[b + 1] - s0;
+    const int32_t t0 = inc_off[v], n = inc_off[v + 1] - t0;
+    for (int k = 0; k < (steps > n ? steps : n); ++k) {
+      int2 q = make_int2(-1, 0);
+      if (k < n) {
+        const int32_t t = t0 + k;
+        q.x = inc[t];
+        uint32_t w = 0;
+        const int32_t tile = (q.x / NV) >> 5;
 #pragma unroll
-        for (int k = 0; k < NV; ++k) wd |= uint32_t(runi[lane * NV + k]) << (8 * k);
+        for (int j = 0; j < NV; ++j) {
+          const uint32_t c = colpos[int64_t(t) * NV + j];
+          uint32_t m = c & 0x3Fu;  // rows of more columns take the scanning path
+          if constexpr (B == 1) {
+            bool first = true, last = true;
+            for (int32_t u = t - 1; first && u >= t0 && (inc[u] / NV) >> 5 == tile; --u)
+#pragma unroll
+              for (int i = 0; i < NV; ++i) first &= colpos[int64_t(u) * NV + i] != c;
+            for (int32_t u = t + 1; last && u < t0 + n && (inc[u] / NV) >> 5 == tile; ++u)
+#pragma unroll
+              for (int i = 0; i < NV; ++i) last &= colpos[int64_t(u) * NV + i] != c;
+            m |= (first ? kFirst : 0u) | (last ? kLast : 0u);
+            nrec += first;
+          }
+          w |= m << (8 * j);
+        }
+        q.y = int(w);
       }
-      run_word[t * 32 + lane] = wd;
-      if (lane == 0) tile_runs[t] = uint16_t(nr | (shared ? 0 : kHalvesDisjoint));
+      if (room && k < steps) slots[(int64_t(s0) + k) * G + (v - b * G)] = q;
     }
-    __syncwarp();  // the buffers are refilled for the next tile
+  }
+  if constexpr (B == 1) {
+    __syncwarp();
+    nrec = __reduce_add_sync(0xffffffffu, nrec);
+    if (nrec && (threadIdx.x & 31) == 0) atomicAdd(n_records, nrec);
   }
 }
 
-// Step 1 of the scalar assembly: one warp per tile, pipelined over its tiles.
-// The next tile's element matrices arrive by 16-byte cp.async into the other
-// half of a double-buffered stage while this tile is summed.  Every lane
-// first writes its element's cell indices (cells[l][ij], shared memory); the
-// dense tile is zero at the start of every tile (zeroed once, and each record
-// cell zeroed again as it is read out); then the contributions are added
-// element by element (each element's cells are distinct) -- two elements per
-// step, l and l + 16, when the tile's halves share no cell -- and the records
-// are read out in tile order.
-template <int NV>
-struct TilePlan {
-  static constexpr int NN = NV * NV;
-  static constexpr int SST = NV == 4 ? 16 : NN;                      // stage row (floats)
-  static constexpr size_t stage = size_t(32) * SST * 4;              // one tile of A
-  static constexpr size_t rcell = size_t(kCellCap) * 2;              // one tile's record cells
-  static constexpr size_t cells = size_t(32) * 17 * 4;               // u32 [32][17]: odd stride, no conflicts
-  static constexpr size_t dense = size_t(kTileRuns) * kTileRuns * 4;
-  static constexpr size_t per_warp = 2 * stage + 2 * rcell + cells + dense;
-  static constexpr size_t smem = kTileWarps * per_warp;
+// Shared memory of a warp: [sums][open tile sums, scalar forms][stage].  The
+// sum of column c of lane l lies at c * 32 + l, a lane's sums in its own bank.
+// Padded slots add zeros to a column of their own (kPadCol), which keeps the
+// loop free of branches.
+//
+// Scalar forms: the element rows come through a stage of two batches of two
+// steps with 16-byte cp.async, which goes around L1.  A scattered load takes a
+// 128-byte line of L1 for every 16 bytes in flight, and beside 200 KB of
+// shared memory L1 has few: with register loads the kernel was bound by them
+// (lanes 31.9 of 32 active, shared-memory pipe 53% busy, waiting on its queue;
+// 96^3 cube 253 us against 134 us with the stage; batches of 1, 4 or 8 steps,
+// or three and four batches, 136 to 160 us).  A lane copies and reads only its
+// own pieces, so no barrier is needed.
+// Blocks: neighbouring lanes read 48 contiguous bytes and half the sums'
+// space, so register loads win (56^3 cube 149 us against 164 us staged); with
+// 8 steps in flight and four CTAs per SM the rest of L1 keeps the sectors that
+// a later row needs (four steps and eight CTAs: 162 us; on triangles the
+// shorter rows prefer the latter, 42 against 46 us at 600 x 600).
+constexpr int kPadCol = kFastCols;
+template <int B>
+struct BlockPlan {
+  static constexpr bool staged = B == 1;
+  static constexpr int warps = staged ? 1 : 4;
+  static constexpr int min_ctas = staged ? 1 : B == 3 ? 4 : 8;
+  static constexpr int batch = staged ? 2 : B == 3 ? 8 : 4;  // steps loaded together
+  static constexpr int stages = staged ? 2 : 1;
+  static constexpr size_t sums = size_t(kFastCols + 1) * 128;
+  static constexpr size_t stage_off = (B == 1 ? 2 : 1) * sums;
+  static constexpr size_t per_warp = stage_off + (staged ? size_t(stages) * batch * 512 : 0);
+  static constexpr size_t smem = warps * per_warp;
 };
 
+// Copies a lane's piece of an element row (NV floats) into its 16 stage bytes; zeros for a padded slot.
 template <int NV>
-__device__ __forceinline__ void copy_tile_A(const float* A, int64_t n_elem, int64_t t, int lane, float* dst,
-                                            int vec) {
-  constexpr int NN = NV * NV;
-  const int64_t e0 = t * 32;
-  if (e0 >= n_elem) return;
-  const int ne = int(n_elem - e0 < 32 ? n_elem - e0 : 32);
-  const float* src = A + e0 * NN;
-  if constexpr (NV == 4) {
-    if (vec) {  // 64-byte rows of a 16-byte-aligned A: contiguous 16-byte chunks
-      for (int q = lane; q < ne * 4; q += 32) cp_async<16>(dst + 4 * q, src + 4 * q);
-      return;
-    }
+__device__ __forceinline__ void copy_piece(void* dst, const float* A, int64_t off, bool real, int vec) {
+  const float* src = real ? A + off : A;
+  if (NV == 4 && vec) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(real ? 16 : 0)
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem_u32(static_cast<float*>(dst) + j)),
+                   "l"(src + (real ? j : 0)), "r"(real ? 4 : 0)
+                   : "memory");
   }
-  for (int q = lane; q < ne * NN; q += 32) cp_async<4>(dst + q, src + q);
 }
 
-// The first rn record cells of tile t (16-byte chunks of its 512-entry slot).
-__device__ __forceinline__ void copy_tile_cells(const uint16_t* rec_cell, int64_t t, int rn, int lane, uint16_t* dst) {
-  const uint16_t* src = rec_cell + t * kCellCap;
-  for (int q = lane; q < (rn + 7) / 8; q += 32) cp_async<16>(dst + 8 * q, src + 8 * q);
-}
-
-template <int NV>
-__global__ void __launch_bounds__(kTileWarps * 32)
-    tile_assemble_kernel(const float* __restrict__ A, int64_t n_elem, const uint32_t* __restrict__ run_word,
-                         const uint16_t* __restrict__ tile_runs, const int32_t* __restrict__ tile_rec,
-                         const uint16_t* __restrict__ rec_cell, const int32_t* __restrict__ rec_dest,
-                         float* __restrict__ records, int vec) {
-  using TP = TilePlan<NV>;
-  constexpr int NN = TP::NN, SST = TP::SST;
-  extern __shared__ __align__(128) unsigned char tsm[];
+// One warp per row block: 32 rows of a scalar form, 8 of 2 x 2 blocks, 3 of
+// 3 x 3 blocks; lane g * B^2 + q serves component q of row g.  A row kernel
+// and not a tile pass with records per entry, because its traffic is one read
+// of A, 8 bytes per incidence and the values (108 bytes per tet of a scalar
+// form, against 197 with records), and because a lane's sums need neither
+// atomics nor barriers.  Scalar forms, 96^3 cube: 241 us (tile pass 190 and
+// entry pass 48) -> 134 us; elasticity, 56^3 cube: 517 us (a thread per row,
+// 5.5 warps per SM) -> 149 us, 4.8 TB/s of the bytes it cannot do without.
+// What bounds it: the L1 and shared-memory pipe (two or three conflict-free
+// accesses a contribution, and a tag look-up per element row).
+template <int NV, int B>
+__global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ctas)
+    assemble_blocks_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                           const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
+                           const int32_t* __restrict__ blk_off, const int2* __restrict__ slots, int64_t slot_cap,
+                           const float* __restrict__ A, int64_t n_vert, float* __restrict__ val, int vec_A) {
+  using BP = BlockPlan<B>;
+  constexpr int BB = B * B, G = block_rows(B), N = NV * B, U = BP::batch;
+  extern __shared__ __align__(128) unsigned char block_sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* wb = tsm + size_t(warp) * TP::per_warp;
-  float* stage = reinterpret_cast<float*>(wb);                                   // [2][32][SST]
-  uint16_t* rcs = reinterpret_cast<uint16_t*>(wb + 2 * TP::stage);               // [2][512]
-  uint32_t* cells = reinterpret_cast<uint32_t*>(wb + 2 * TP::stage + 2 * TP::rcell);
-  float* dense = reinterpret_cast<float*>(wb + 2 * TP::stage + 2 * TP::rcell + TP::cells);
-  const int64_t ntiles = (n_elem + 31) / 32;
-  const int64_t S = int64_t(gridDim.x) * kTileWarps;
-  int64_t t = int64_t(blockIdx.x) * kTileWarps + warp;
-  if (t >= ntiles) return;
-  // pipeline: tile metadata two tiles ahead, A / record cells / runs one tile ahead
-  auto meta = [&](int64_t tt, int& tr, int32_t& rb, int32_t& rn) {
-    tr = 0, rb = 0, rn = 0;
-    if (tt < ntiles) {
-      tr = __ldg(tile_runs + tt);
-      rb = __ldg(tile_rec + tt);
-      rn = __ldg(tile_rec + tt + 1) - rb;
-    }
-  };
-  int trc, trn, tr2;
-  int32_t rbc, rnc, rbn, rnn, rb2, rn2;
-  meta(t, trc, rbc, rnc);
-  meta(t + S, trn, rbn, rnn);
-  copy_tile_A<NV>(A, n_elem, t, lane, stage, vec);
-  copy_tile_cells(rec_cell, t, rnc, lane, rcs);
-  cp_async_commit();
-  uint32_t rwc = __ldg(run_word + t * 32 + lane);
-  // the entry-order slots of a tile's first 32 * kDestRegs records, one tile ahead
-  auto dests = [&](int32_t rb, int32_t rn, int32_t(&d)[kDestRegs]) {
+  unsigned char* wbase = block_sm + size_t(warp) * BP::per_warp;
+  float* tot = reinterpret_cast<float*>(wbase);
+  char* mine = reinterpret_cast<char*>(wbase) + 4 * lane;
+  char* stage = reinterpret_cast<char*>(wbase) + BP::stage_off + 16 * lane;
+  constexpr int kPart = int(BP::sums);     // from a sum to the open tile sum
+  const int g = lane / BB, q = lane % BB;  // row of the block, component (c, c2) = (q / B, q % B)
+  // offset of the component's row and columns in A_e, without the element slot
+  const float* Aq = A + (B == 1 ? 0 : (q / B) * NV * N + (q % B) * NV);
+  const int64_t nblk = (n_vert + G - 1) / G;
+  const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
+  // the sums are zero at the start of every block: zeroed here, and again as they are read out
+  for (int c = 0; c <= kFastCols; ++c) *reinterpret_cast<float*>(mine + c * 128) = 0.f;
+  for (int64_t b = int64_t(blockIdx.x) * BP::warps + warp; b < nblk; b += int64_t(gridDim.x) * BP::warps) {
+    const int64_t r0 = b * G;
+    const int nr = int(n_vert - r0 < G ? n_vert - r0 : G);
+    const int32_t s0 = __ldg(blk_off + b), steps = __ldg(blk_off + b + 1) - s0;
+    const int32_t rp0 = __ldg(row_ptr + r0), total = __ldg(row_ptr + r0 + nr) - rp0;
+    if (total == 0) continue;
+    if (room && steps > 0) {
+      const bool live = g < nr;
+      const int32_t rb = live ? __ldg(row_ptr + r0 + g) : 0;
+      const int len = live ? __ldg(row_ptr + r0 + g + 1) - rb : 0;
+      const int2* sl = slots + int64_t(s0) * G + g;
+      int2 ahead[U];  // slots of the next batch to load
+      auto load_slots = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < kDestRegs; ++q) d[q] = lane + 32 * q < rn ? __ldg(rec_dest + rb + lane + 32 * q) : 0;
-  };
-  int32_t dc[kDestRegs], dn[kDestRegs];
-  dests(rbc, rnc, dc);
-  for (int i = lane; i < kTileRuns * kTileRuns; i += 32) dense[i] = 0.f;
-  for (int it = 0; t < ntiles; ++it, t += S) {
-    const int sc = it & 1;
-    const int64_t tn = t + S;
-    meta(tn + S, tr2, rb2, rn2);
-    uint32_t rwn = 0;
-    if (tn < ntiles) {
-      copy_tile_A<NV>(A, n_elem, tn, lane, stage + (sc ^ 1) * 32 * SST, vec);
-      copy_tile_cells(rec_cell, tn, rnn, lane, rcs + (sc ^ 1) * kCellCap);
-      rwn = __ldg(run_word + tn * 32 + lane);
-    }
-    dests(rbn, rnn, dn);  // rnn = 0 past the last tile
-    cp_async_commit();
-    const int64_t e0 = t * 32;
-    const int ne = int(n_elem - e0 < 32 ? n_elem - e0 : 32);
-    const int nr = trc & 0xFF;
-    const bool halves = (trc & kHalvesDisjoint) && ne == 32;
-    const float* st = stage + sc * 32 * SST;
-    const uint16_t* rc = rcs + sc * kCellCap;
-    const uint32_t ps = uint32_t(cell_stride(nr));
-    if (nr <= kTileRuns && lane < ne) {
+        for (int u = 0; u < U; ++u)
+          ahead[u] = live && k0 + u < steps ? __ldg(sl + (k0 + u) * G) : make_int2(-1, kPadCol * 0x01010101);
+      };
+      // row (c, i) of A_e, columns (c2, 0 .. NV-1): for tets 16 bytes at a multiple of 16
+      auto piece = [&](int32_t s) {
+        return B == 1 ? int64_t(s) * NV : int64_t(s / NV) * (N * N) + (s % NV) * N;
+      };
+      // adds a step's piece; its NV columns differ (or are all the pad column): read all, add, write all
+      auto add_step = [&](const float(&a)[4], uint32_t w) {
+        char* at[NV];
+        float s[NV], o[NV];
 #pragma unroll
-      for (int ij = 0; ij < NN; ++ij)
-        cells[lane * 17 + ij] = ((rwc >> (8 * (ij / NV))) & 0xFFu) * ps + ((rwc >> (8 * (ij % NV))) & 0xFFu);
-    }
-    cp_async_wait<1>();
-    __syncwarp();  // this tile's A and record cells (copied by every lane) and the cell indices are in place
-    if (nr <= kTileRuns) {
-      if (halves) {
-        const int h = lane >> 4, ij = lane & 15;
-        for (int l0 = 0; l0 < 16; ++l0) {
-          const int l = l0 + 16 * h;
-          if (ij < NN) dense[cells[l * 17 + ij]] += st[l * SST + ij];
-          __syncwarp();
+        for (int j = 0; j < NV; ++j) at[j] = mine + ((j == 0 ? w << 7 : w >> (8 * j - 7)) & (0x3Fu << 7));
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          s[j] = *reinterpret_cast<float*>(at[j]);
+          if (B == 1) o[j] = *reinterpret_cast<float*>(at[j] + kPart);
         }
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          if constexpr (B == 1) {
+            const bool first = w & (kFirst << (8 * j)), last = w & (kLast << (8 * j));
+            float r = (first ? 0.f : o[j]) + a[j];
+            if (last) r = s[j] + r;
+            *reinterpret_cast<float*>(at[j] + (last ? 0 : kPart)) = r;
+          } else {
+            *reinterpret_cast<float*>(at[j]) = s[j] + a[j];
+          }
+        }
+      };
+      load_slots(0);
+      if constexpr (BP::staged) {
+        constexpr int S = BP::stages;
+        uint32_t word[S][U];  // column words of the batches in flight
+        auto copy_batch = [&](int st) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            copy_piece<NV>(stage + (st * U + u) * 512, Aq, piece(ahead[u].x), ahead[u].x >= 0, vec_A);
+            word[st][u] = uint32_t(ahead[u].y);
+          }
+          cp_async_commit();
+        };
+#pragma unroll
+        for (int st = 0; st < S - 1; ++st) {
+          copy_batch(st);
+          load_slots((st + 1) * U);
+        }
+        for (int k0 = 0; k0 < steps; k0 += S * U)
+#pragma unroll
+          for (int st = 0; st < S; ++st) {  // the batch at k0 + st * U, in stage st
+            copy_batch(st == 0 ? S - 1 : st - 1);
+            load_slots(k0 + (st + S) * U);
+            cp_async_wait<S - 1>();
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const float4 v = *reinterpret_cast<const float4*>(stage + (st * U + u) * 512);
+              add_step({v.x, v.y, v.z, v.w}, word[st][u]);
+            }
+          }
+        cp_async_wait<0>();
       } else {
-        for (int l = 0; l < ne; ++l) {  // element order
-          if (lane < NN) dense[cells[l * 17 + lane]] += st[l * SST + lane];
-          __syncwarp();
-        }
-      }
+        for (int k0 = 0; k0 < steps; k0 += U) {
+          float a[U][4];
+          uint32_t word[U];
 #pragma unroll
-      for (int q = 0; q < kDestRegs; ++q)
-        if (lane + 32 * q < rnc) {
-          const int c = rc[lane + 32 * q];
-          records[dc[q]] = dense[c];
-          dense[c] = 0.f;
+          for (int u = 0; u < U; ++u) {
+            const float* src = Aq + piece(ahead[u].x);
+            word[u] = uint32_t(ahead[u].y);
+#pragma unroll
+            for (int j = 0; j < NV; ++j) a[u][j] = 0.f;
+            if (ahead[u].x >= 0) {
+              if (NV == 4 && vec_A) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+                a[u][0] = v.x, a[u][1] = v.y, a[u][2] = v.z, a[u][3] = v.w;
+              } else {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) a[u][j] = __ldg(src + j);
+              }
+            }
+          }
+          load_slots(k0 + U);
+#pragma unroll
+          for (int u = 0; u < U; ++u) add_step(a[u], word[u]);
         }
-      for (int r = lane + 32 * kDestRegs; r < rnc; r += 32) {
-        const int c = rc[r];
-        records[__ldg(rec_dest + rbc + r)] = dense[c];
-        dense[c] = 0.f;
       }
+      const int maxlen = __reduce_max_sync(0xffffffffu, len);
+      if constexpr (B == 1) {
+        // pack the rows' values where the open tile sums were (all closed) and store them coalesced
+        __syncwarp();
+        float* pack = reinterpret_cast<float*>(wbase + kPart);
+        for (int c = 0; c < maxlen; ++c)
+          if (c < len) {
+            float* w = reinterpret_cast<float*>(mine + c * 128);
+            pack[rb - rp0 + c] = *w;
+            *w = 0.f;
+          }
+        __syncwarp();
+        for (int x = lane; x < total; x += 32) __stcs(val + int64_t(rp0) + x, pack[x]);
+      } else {
+        // a lane's values straight from its bank: 36 (16) contiguous bytes per row and column
+        float* out = val + int64_t(rb) * BB + q;
+        for (int c = 0; c < maxlen; ++c)
+          if (c < len) {
+            float* w = reinterpret_cast<float*>(mine + c * 128);
+            out[c * BB] = *w;
+            *w = 0.f;
+          }
+      }
+      __syncwarp();  // the sums are the next block's
     } else {
-      // more distinct vertices than the dense tile holds: scan the tile per record
-      for (int r0 = 0; r0 < rnc; r0 += 32) {  // warp-uniform, so the shuffles see every lane
-        const int r = r0 + lane;
-        const bool live = r < rnc;
-        const int cell = live ? int(rc[r]) : -1;
-        float acc = 0.f;
-        for (int l = 0; l < ne; ++l) {
-          const uint32_t w = __shfl_sync(0xffffffffu, rwc, l);
+      // scanning path: a lane per value, every incidence of the row looked at
+      for (int h = 0; h < nr; ++h) {
+        const int32_t rp = __ldg(row_ptr + r0 + h), t0 = __ldg(inc_off + r0 + h), t1 = __ldg(inc_off + r0 + h + 1);
+        const int words = (__ldg(row_ptr + r0 + h + 1) - rp) * BB;
+        for (int x = lane; x < words; x += 32) {
+          const int c = x / BB, c1 = (x % BB) / B, c2 = x % B;
+          float sum = 0.f, part = 0.f;
+          int tile = -1;
+          for (int32_t t = t0; t < t1; ++t) {
+            const int32_t s = __ldg(inc + t);
+            const float* src = A + int64_t(s / NV) * (N * N) + (c1 * NV + s % NV) * N + c2 * NV;
+            if (B == 1 && (s / NV) >> 5 != tile) {
+              sum += part;
+              part = 0.f;
+              tile = (s / NV) >> 5;
+            }
 #pragma unroll
-          for (int ij = 0; ij < NN; ++ij)
-            if (int((w >> (8 * (ij / NV))) & 0xFFu) * int(ps) + int((w >> (8 * (ij % NV))) & 0xFFu) == cell)
-              acc += st[l * SST + ij];
+            for (int j = 0; j < NV; ++j)
+              if (__ldg(colpos + int64_t(t) * NV + j) == c) (B == 1 ? part : sum) += __ldg(src + j);
+          }
+          val[int64_t(rp) * BB + x] = sum + part;
         }
-        if (live) records[__ldg(rec_dest + rbc + r)] = acc;
       }
     }
-    __syncwarp();  // the stage, record cells, cells and dense tile are refilled
-    trc = trn, rbc = rbn, rnc = rnn, rwc = rwn;
-#pragma unroll
-    for (int q = 0; q < kDestRegs; ++q) dc[q] = dn[q];
-    trn = tr2, rbn = rb2, rnn = rn2;
-  }
-  cp_async_wait<0>();
-}
-
-// Step 2: val[k] = sum of the records of entry k, records[eoff[k] .. eoff[k+1])
-// in tile order: the tile pass wrote every record to its slot in entry order,
-// so neighbouring threads read neighbouring runs.  A thread sums two entries
-// at a time (k and k + S), four records of each loaded before they are added,
-// while the bounds of its next two entries load.
-__global__ void entry_reduce_kernel(const int32_t* __restrict__ eoff, const int32_t* __restrict__ nnz_ptr,
-                                    const float* __restrict__ records, float* __restrict__ val) {
-  const int64_t nnz = *nnz_ptr;  // row_ptr[n_vert]
-  const int64_t S = int64_t(gridDim.x) * blockDim.x;
-  auto bounds = [&](int64_t k, int32_t& b, int32_t& e) {
-    b = 0, e = 0;
-    if (k < nnz) b = __ldg(eoff + k), e = __ldg(eoff + k + 1);
-  };
-  int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  int32_t b0n, e0n, b1n, e1n;
-  bounds(k, b0n, e0n);
-  bounds(k + S, b1n, e1n);
-  for (; k < nnz; k += 2 * S) {
-    const int32_t b0 = b0n, e0 = e0n, b1 = b1n, e1 = e1n;
-    bounds(k + 2 * S, b0n, e0n);
-    bounds(k + 3 * S, b1n, e1n);
-    const int32_t n0 = e0 - b0, n1 = e1 - b1;
-    float acc0 = 0.f, acc1 = 0.f;
-    for (int32_t m0 = 0; m0 < n0 || m0 < n1; m0 += 4) {
-      float x0[4], x1[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        x0[u] = m0 + u < n0 ? __ldg(records + b0 + m0 + u) : 0.f;
-        x1[u] = m0 + u < n1 ? __ldg(records + b1 + m0 + u) : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (m0 + u < n0) acc0 += x0[u];
-        if (m0 + u < n1) acc1 += x1[u];
-      }
-    }
-    val[k] = acc0;
-    if (k + S < nnz) val[k + S] = acc1;
   }
 }
 
 struct AsmLayout {
-  int32_t *inc_off, *inc, *row_ptr, *col_idx, *cursor, *partials, *flag;
+  int32_t *inc_off, *inc, *row_ptr, *col_idx, *cursor, *partials;
+  int32_t* flag;  // [0] build flags, [1] tile records (scalar forms)
   uint8_t* colpos;
-  // tile records (scalar forms)
-  uint32_t* run_word;
-  uint16_t* tile_runs;
-  int32_t *tile_rec, *rec_entry, *rec_list, *eoff, *cursor2, *partials2;
-  int32_t* rec_dest;  // the records' entry-order slots; shares rec_entry's storage, which the build no longer needs
-  uint16_t* rec_cell;
-  float* records;
-  int64_t n_tiles, rec_cap;
+  // row blocks (P1 forms and elasticity)
+  int32_t* blk_off;  // [blocks + 1] first step of each block
+  int2* slots;       // [steps][block_rows]: (element slot or -1, column word)
+  int64_t slot_cap;
   size_t bytes;
 };
 
@@ -610,34 +485,28 @@ size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 AsmLayout asm_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
   const int64_t nv = dim + 1;
-  const int64_t T = (n_elem + 31) / 32;
-  const int64_t cap = n_elem * nv * nv;  // contributions: bounds the entries and the records
-  const int64_t big = (T > cap ? T : cap) + 1;
+  const int64_t cap = n_elem * nv * nv;  // contributions: bounds the entries
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off = al256(off + bytes);
     return o;
   };
+  AsmLayout L{};
+  // Room for padding the rows of a block to its longest one: twice the
+  // incidences (a cube's rows need 1.1 times; a mesh that needs more than
+  // twice takes the scanning path of the kernel, which reads no slots).
+  L.slot_cap = 2 * n_elem * nv + 1024;
   const size_t o_inc_off = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_inc = take(sizeof(int32_t) * size_t(n_elem * nv));
-  const size_t o_colpos = take(size_t(n_elem * nv * nv));
+  const size_t o_colpos = take(size_t(cap));
   const size_t o_row_ptr = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_col = take(sizeof(int32_t) * size_t(cap));  // capacity: every entry distinct
   const size_t o_cursor = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_part = take(sizeof(int32_t) * scan_partials_count(n_vert + 1));
   const size_t o_flag = take(sizeof(int32_t) * 4);
-  const size_t o_run = take(sizeof(uint32_t) * size_t(T * 32));
-  const size_t o_truns = take(sizeof(uint16_t) * size_t(T));
-  const size_t o_trec = take(sizeof(int32_t) * size_t(T + 1));
-  const size_t o_cell = take(sizeof(uint16_t) * size_t(T * kCellCap));  // 512 cells per tile, tile-strided
-  const size_t o_rentry = take(sizeof(int32_t) * size_t(cap));
-  const size_t o_rlist = take(sizeof(int32_t) * size_t(cap));
-  const size_t o_eoff = take(sizeof(int32_t) * size_t(cap + 1));
-  const size_t o_records = take(sizeof(float) * size_t(cap));
-  const size_t o_cursor2 = take(sizeof(int32_t) * size_t(big));
-  const size_t o_part2 = take(sizeof(int32_t) * scan_partials_count(big));
-  AsmLayout L{};
+  const size_t o_blk = take(sizeof(int32_t) * size_t(n_vert + 2));
+  const size_t o_slots = take(sizeof(int2) * size_t(L.slot_cap));
   char* b = static_cast<char*>(base);
   L.inc_off = reinterpret_cast<int32_t*>(b + o_inc_off);
   L.inc = reinterpret_cast<int32_t*>(b + o_inc);
@@ -647,34 +516,10 @@ AsmLayout asm_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
   L.cursor = reinterpret_cast<int32_t*>(b + o_cursor);
   L.partials = reinterpret_cast<int32_t*>(b + o_part);
   L.flag = reinterpret_cast<int32_t*>(b + o_flag);
-  L.run_word = reinterpret_cast<uint32_t*>(b + o_run);
-  L.tile_runs = reinterpret_cast<uint16_t*>(b + o_truns);
-  L.tile_rec = reinterpret_cast<int32_t*>(b + o_trec);
-  L.rec_cell = reinterpret_cast<uint16_t*>(b + o_cell);
-  L.rec_entry = reinterpret_cast<int32_t*>(b + o_rentry);
-  L.rec_list = reinterpret_cast<int32_t*>(b + o_rlist);
-  L.rec_dest = L.rec_entry;
-  L.eoff = reinterpret_cast<int32_t*>(b + o_eoff);
-  L.records = reinterpret_cast<float*>(b + o_records);
-  L.cursor2 = reinterpret_cast<int32_t*>(b + o_cursor2);
-  L.partials2 = reinterpret_cast<int32_t*>(b + o_part2);
-  L.n_tiles = T;
-  L.rec_cap = cap;
+  L.blk_off = reinterpret_cast<int32_t*>(b + o_blk);
+  L.slots = reinterpret_cast<int2*>(b + o_slots);
   L.bytes = off;
   return L;
-}
-
-// rec_dest[rec_list[p]] = p for the *n_rec records listed
-__global__ void invert_list_kernel(const int32_t* __restrict__ rec_list, const int32_t* __restrict__ n_rec,
-                                   int32_t* __restrict__ rec_dest) {
-  const int64_t n = *n_rec;
-  for (int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; p < n; p += int64_t(gridDim.x) * blockDim.x)
-    rec_dest[rec_list[p]] = int32_t(p);
-}
-
-__global__ void fill_neg_kernel(int32_t* p, int64_t n) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    p[i] = -1;
 }
 
 unsigned grid_of(int64_t n, int per_block) {
@@ -696,44 +541,31 @@ cudaError_t launch_pattern(int dim, const int32_t* conn, int64_t n_vert, const A
   return cudaGetLastError();
 }
 
-template <bool WRITE>
-cudaError_t launch_tile_cells(int dim, const int32_t* conn, int64_t n_elem, const AsmLayout& L, cudaStream_t st) {
-  const unsigned g = grid_of(L.n_tiles, kPatWarps);
-  if (dim == 2)
-    tile_cells_kernel<3, WRITE><<<g, kPatWarps * 32, 0, st>>>(conn, n_elem, L.row_ptr, L.col_idx, L.cursor2,
-                                                               L.tile_rec, L.run_word, L.tile_runs, L.rec_cell,
-                                                               L.rec_entry, L.flag);
-  else
-    tile_cells_kernel<4, WRITE><<<g, kPatWarps * 32, 0, st>>>(conn, n_elem, L.row_ptr, L.col_idx, L.cursor2,
-                                                               L.tile_rec, L.run_word, L.tile_runs, L.rec_cell,
-                                                               L.rec_entry, L.flag);
-  return cudaGetLastError();
-}
-
-template <int NV>
-cudaError_t launch_tile_assemble_t(const AsmLayout& L, const float* A, int64_t n_elem, int64_t n_vert, float* val,
-                                   cudaStream_t st) {
-  const size_t smem = TilePlan<NV>::smem;
-  auto kern = tile_assemble_kernel<NV>;
-  cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
+// The row blocks of a built pattern (B = block size of the form).  Scalar
+// forms also count their tile records into L.flag[1].
+template <int NV, int B>
+cudaError_t launch_row_blocks(int64_t n_vert, const AsmLayout& L, cudaStream_t st) {
+  const int64_t nblk = (n_vert + block_rows(B) - 1) / block_rows(B);
+  block_steps_kernel<NV, B><<<grid_of(nblk, 256), 256, 0, st>>>(L.inc_off, L.row_ptr, L.colpos, n_vert, L.cursor);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_exclusive_scan(L.cursor, nblk, L.partials, L.blk_off, st);
   if (e != cudaSuccess) return e;
-  kern<<<pipeline_grid(reinterpret_cast<const void*>(kern), kTileWarps, smem, n_elem, 0), kTileWarps * 32, smem, st>>>(
-      A, n_elem, L.run_word, L.tile_runs, L.tile_rec, L.rec_cell, L.rec_dest, L.records,
-      int(reinterpret_cast<uintptr_t>(A) % 16 == 0));
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  entry_reduce_kernel<<<grid_of(L.rec_cap, 256), 256, 0, st>>>(L.eoff, L.row_ptr + n_vert, L.records, val);
+  block_fill_kernel<NV, B><<<grid_of(n_vert, 256), 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.blk_off, n_vert,
+                                                                 L.slot_cap, L.slots, L.flag + 1);
   return cudaGetLastError();
 }
 
 template <int NV, int B>
 cudaError_t launch_assemble_t(const AsmLayout& L, const float* A, int64_t n_vert, float* val, cudaStream_t st) {
-  const size_t smem = size_t(kAsmThreads) * (kFastCols * B * B + 1) * sizeof(float);
-  auto kern = assemble_kernel<NV, B>;
-  cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
+  auto kern = assemble_blocks_kernel<NV, B>;
+  constexpr int warps = BlockPlan<B>::warps;
+  constexpr size_t smem = BlockPlan<B>::smem;
+  const cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  const int vec_A = reinterpret_cast<uintptr_t>(A) % 16 == 0;
-  kern<<<grid_of(n_vert, kAsmThreads), kAsmThreads, smem, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, A, n_vert,
-                                                                 val, vec_A, nullptr);
+  const int64_t nblk = (n_vert + block_rows(B) - 1) / block_rows(B);
+  const unsigned g = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, nblk * 32, 0);
+  kern<<<g, warps * 32, smem, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off, L.slots, L.slot_cap, A, n_vert,
+                                    val, int(reinterpret_cast<uintptr_t>(A) % 16 == 0));
   return cudaGetLastError();
 }
 
@@ -1112,27 +944,25 @@ fem_status fem_assembly_build(const fem_mesh* mesh, int32_t form, void* ws, size
   if (e == cudaSuccess && V > 0) e = fem::launch_pattern<false>(mesh->dim, mesh->conn, V, L, st);
   if (e == cudaSuccess) e = fem::launch_exclusive_scan(L.cursor, V, L.partials, L.row_ptr, st);
   if (e == cudaSuccess && V > 0) e = fem::launch_pattern<true>(mesh->dim, mesh->conn, V, L, st);
+  const int B = asm_block(form, mesh->dim);
+  if (e == cudaSuccess && B == 1 && mesh->n_elem > 0) {  // the scalar forms refuse an element repeating a vertex
+    const unsigned g = fem::grid_of(mesh->n_elem, 256);
+    if (mesh->dim == 2)
+      fem::check_repeat_kernel<3><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, L.flag);
+    else
+      fem::check_repeat_kernel<4><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, L.flag);
+    e = cudaGetLastError();
+  }
   int32_t host[2] = {0, 0}, nrec = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&host[0], L.flag, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&host[1], L.row_ptr + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  // tile records of the scalar forms: cells per 32-element tile, entry-major records
-  if (e == cudaSuccess && host[0] == 0 && asm_block(form, mesh->dim) == 1 && mesh->n_elem > 0) {
-    e = fem::launch_tile_cells<false>(mesh->dim, mesh->conn, mesh->n_elem, L, st);
-    if (e == cudaSuccess) e = fem::launch_exclusive_scan(L.cursor2, L.n_tiles, L.partials2, L.tile_rec, st);
-    if (e == cudaSuccess) {
-      fem::fill_neg_kernel<<<fem::grid_of(L.rec_cap, 256), 256, 0, st>>>(L.rec_entry, L.rec_cap);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = fem::launch_tile_cells<true>(mesh->dim, mesh->conn, mesh->n_elem, L, st);
-    if (e == cudaSuccess)
-      e = fem::launch_key_csr(L.rec_entry, L.rec_cap, host[1], L.eoff, L.rec_list, L.cursor2, L.partials2, st);
-    if (e == cudaSuccess) {  // eoff[nnz] = the records
-      fem::invert_list_kernel<<<fem::grid_of(L.rec_cap, 256), 256, 0, st>>>(L.rec_list, L.eoff + host[1], L.rec_dest);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&host[0], L.flag, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nrec, L.tile_rec + L.n_tiles, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && host[0] == 0 && V > 0) {
+    if (mesh->dim == 2)
+      e = B == 1 ? fem::launch_row_blocks<3, 1>(V, L, st) : fem::launch_row_blocks<3, 2>(V, L, st);
+    else
+      e = B == 1 ? fem::launch_row_blocks<4, 1>(V, L, st) : fem::launch_row_blocks<4, 3>(V, L, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&nrec, L.flag + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
   if (e != cudaSuccess) {
@@ -1207,15 +1037,15 @@ fem_status fem_assemble(const fem_mesh* mesh, int32_t form, const float* A, cons
   if (asm_p2(form)) {  // the row kernel over the vertex and edge unknowns
     const fem::AsmP2Layout P = fem::asm_p2_layout(mesh->dim, mesh->n_elem, mesh->n_vert, const_cast<void*>(ws));
     e = mesh->dim == 2 ? fem::launch_p2_assemble<6>(P, A, values, st) : fem::launch_p2_assemble<10>(P, A, values, st);
-  } else if (B == 1 && mesh->n_elem > 0)  // scalar forms: tile records, then the per-entry sums
-    e = mesh->dim == 2 ? fem::launch_tile_assemble_t<3>(L, A, mesh->n_elem, mesh->n_vert, values, st)
-                       : fem::launch_tile_assemble_t<4>(L, A, mesh->n_elem, mesh->n_vert, values, st);
-  else if (mesh->dim == 2)
+  } else if (mesh->n_elem == 0) {
+    return FEM_OK;
+  } else if (mesh->dim == 2) {
     e = B == 1 ? fem::launch_assemble_t<3, 1>(L, A, mesh->n_vert, values, st)
                : fem::launch_assemble_t<3, 2>(L, A, mesh->n_vert, values, st);
-  else
+  } else {
     e = B == 1 ? fem::launch_assemble_t<4, 1>(L, A, mesh->n_vert, values, st)
                : fem::launch_assemble_t<4, 3>(L, A, mesh->n_vert, values, st);
+  }
   if (e != cudaSuccess) {
     fem::set_last_error("fem_assemble: %s", cudaGetErrorString(e));
     return FEM_ERR_CUDA;
