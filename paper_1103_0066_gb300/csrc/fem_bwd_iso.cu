@@ -8,9 +8,10 @@
 // (J_c = the mean of the vertex Jacobians, the map being quadratic), and
 //   A_T = scale * sum_g K'[g][T] H_g,   H_g = sum_a ji[k][mu][a] ji[l][nu][a]
 // over the folded slot pairs g = ((k mu), (l nu)).  Per lane, in reverse:
-//   1. s_g = sum_T K'[g][T] sym(dA)_T (the contraction's adjoint, K' as
-//      immediates, one g at a time), dscale += s_g H_g and
-//      dji[k][mu] += scale s_g ji[l][nu] (and symmetrically);
+//   1. the contraction's adjoint by the structure of K (fem_iso_mat.cuh):
+//      the gradient u of sum_T sym(dA)_T A_T / scale with respect to the
+//      inverse Jacobians; dji = scale u, and dscale = sum u . ji / 2, the sum
+//      being homogeneous of degree two;
 //   2. dw = dscale |det J_c| / DEN, d det(e_c) = sgn w dscale / (DEN (d+1)^d),
 //      d e_c = d det(e_c) adj(e_c), added to every d e_k;
 //   3. ji = e^{-T}: d e_k = -ji[k] dji[k]^T ji[k] + d e_c;
@@ -21,27 +22,39 @@
 // coefficient gradients are per element.  The tile's edge nodes come in, and
 // their gradients go out, through a shared-memory stage as contiguous 16-byte
 // pieces (an element's 18 floats are not 16-byte aligned on their own).
+// A warp copies its next tile's dA as soon as every lane holds sym(dA) in
+// registers, so the copy (12.8 of a P2 tet tile's 15 KB of input) runs under
+// the arithmetic; the next connectivity is loaded with it.
+// P2 tets, 64^3 cube: 343 us with the contraction over 78 folded slot pairs,
+// 291 us by the structure of K, 240 us with the copy ahead and 12 warps per SM
+// (8 at the 250 registers it takes unbounded: 244 us; 16 spill: 310 us).
+// Bound by instruction issue and the latency of the geometry's loads (issue
+// 56% active at 11.4 warps).  P1 tets: 102 us.
 #include "fem_iso_adj.cuh"
+#include "fem_iso_mat.cuh"
 
 namespace fem {
 
 namespace {
 
 // CTA shape: one-warp CTAs on tets (no CTA-wide barrier), each holding the
-// four inverse Jacobians, their adjoints and sym(dA) in registers.
+// four inverse Jacobians, their adjoints and sym(dA) in registers: 168 a
+// thread for P2 (104 bytes spilled), three warps on each quarter of an SM.
 template <int D, int FORM>
 struct IsoBwdShape {
   static constexpr int threads = D == 3 ? 32 : kTileElems;
-  static constexpr int min_ctas = D == 3 ? (FORM == LAPLACE_P1_ISO ? 16 : 8) : 1;
+  static constexpr int min_ctas = D == 3 ? (FORM == LAPLACE_P1_ISO ? 16 : 12) : 1;
 };
 
-// Per warp: [dA slot][slot stage][edge nodes of the tile, then their gradients].
+// Per warp: [dA slot][a region that holds the tile's edge nodes, then the slot
+// stage, then the edge-node gradients].
 template <int D, int FORM>
 struct IsoBwdPlan {
   using PL = BwdPlan<D, FORM>;
   static constexpr int NEF = D * D * (D + 1) / 2;  // edge-node floats per element
   static constexpr size_t mid_bytes = align_up(size_t(32) * NEF * 4, 128);
-  static constexpr size_t per_warp = PL::da_slot + PL::xs_bytes + mid_bytes;
+  static constexpr size_t region = mid_bytes > PL::xs_bytes ? mid_bytes : PL::xs_bytes;
+  static constexpr size_t per_warp = PL::da_slot + region;
 };
 
 template <int D, int FORM, bool ATOMIC>
@@ -55,19 +68,24 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
   unsigned char* wbase = smem_raw + size_t(warp) * IsoBwdPlan<D, FORM>::per_warp;
   float* dslot = reinterpret_cast<float*>(wbase);
   float* xs = reinterpret_cast<float*>(wbase + PL::da_slot);
-  float* ms = reinterpret_cast<float*>(wbase + PL::da_slot + PL::xs_bytes);  // [32][NE * D]
+  float* ms = xs;  // [32][NE * D]
   const bool rec = !ATOMIC && p.tile_rec != nullptr;
   const int64_t ntiles = (p.n_elem + 31) / 32;
   int err = 0;
-  for (int64_t t = int64_t(blockIdx.x) * nwarps + warp; t < ntiles; t += int64_t(gridDim.x) * nwarps) {
+  const int64_t S = int64_t(gridDim.x) * nwarps;
+  int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  if (t >= ntiles) return;  // warp-uniform: the kernel has no CTA-wide barrier
+  int v[NV], vn[NV];
+  copy_dA_async<D, FORM>(p, t, lane, dslot);
+  cp_async_commit();
+  load_conn<D>(p.conn, t * 32 + lane, p.n_elem, p.vec_conn, v);
+  for (; t < ntiles; t += S) {
     const int64_t e = t * 32 + lane;
     const int cnt = int(p.n_elem - t * 32 < 32 ? p.n_elem - t * 32 : 32);
-    copy_dA_async<D, FORM>(p, t, lane, dslot);
     tile_load_async(ms, mid + t * 32 * (NE * D), cnt * (NE * D), lane);
     cp_async_commit();
-    int v[NV];
+    load_conn<D>(p.conn, e + S * 32, p.n_elem, p.vec_conn, vn);
     float X[NV][D];
-    load_conn<D>(p.conn, e, p.n_elem, p.vec_conn, v);
     const int flags = gather_regs<D>(p.coords, p.n_vert, e, p.n_elem, v, X);
     uint32_t rk = 0;
     int32_t rb = 0, rn = 0;
@@ -90,11 +108,11 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
     bool ok = false;
     cp_async_wait<0>();
     __syncwarp();  // the tile's dA rows were copied by other lanes
+    // geometry as the forward forms it: nodes relative to vertex 0, J^{-1} at
+    // the vertices, the centroid's edge vectors and adjugate
+    float ji[NV][D][D], adjc[D][D], detc = 0.f;
     if (flags & GF_OK) {
-      const float w = (p.coef && e < p.n_elem) ? __ldg(p.coef + e) : 1.f;
-      // geometry as the forward forms it: nodes relative to vertex 0, J^{-1}
-      // at the vertices, the centroid's edge vectors and adjugate
-      float nd[NG][D];
+      float nd[NG][D], ec[D][D];
 #pragma unroll
       for (int a = 0; a <= D; ++a)
 #pragma unroll
@@ -104,67 +122,74 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
       for (int q = 0; q < NE; ++q)
 #pragma unroll
         for (int al = 0; al < D; ++al) nd[D + 1 + q][al] = me[q * D + al] - X[0][al];
-      float ji[NV][D][D], ec[D][D], adjc[D][D];
       ok = all_vertex_jinv<D>(nd, ji, ec, std::make_integer_sequence<int, NV>{});
-      const float detc = det_adj<D>(ec, adjc) * (D == 2 ? (1.f / 9.f) : (1.f / 64.f));
+      detc = det_adj<D>(ec, adjc) * (D == 2 ? (1.f / 9.f) : (1.f / 64.f));
       ok &= detc != 0.f;
-      if (!ok) {
-        err |= DEVERR_DEGENERATE;
-      } else {
-        const float absdet = fabsf(detc);
-        const float sc = w * absdet * (1.f / float(FT::DEN));
-        // 1. the contraction's adjoint, one folded slot pair at a time
-        float dji[NV][D][D];
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int mu = 0; mu < D; ++mu)
-#pragma unroll
-            for (int a = 0; a < D; ++a) dji[k][mu][a] = 0.f;
-        float dsc = 0.f;
-        {
-          SymVals<FT::NT> sym;
-          stage_sym<D, FORM>(dslot + lane * PL::DST, sym.s);
-          iso_adj_all<D, FORM>(sym, ji, sc, dji, dsc, std::make_integer_sequence<int, FT::NG>{});
-        }
-        // 2. coefficient and centroid determinant
-        dw = dsc * absdet * (1.f / float(FT::DEN));
-        const float ddet = (detc > 0.f ? 1.f : -1.f) * dsc * w * (1.f / float(FT::DEN)) *
-                           (D == 2 ? (1.f / 9.f) : (1.f / 64.f));
-        float dec[D][D];
-#pragma unroll
-        for (int mu = 0; mu < D; ++mu)
-#pragma unroll
-          for (int al = 0; al < D; ++al) dec[mu][al] = ddet * adjc[mu][al];
-        // 3.-4. inverse Jacobians and the centroid term pulled back to the nodes
-        float dnd[NG][D];
-#pragma unroll
-        for (int a = 0; a < NG; ++a)
-#pragma unroll
-          for (int al = 0; al < D; ++al) dnd[a][al] = 0.f;
-        all_vertex_pullback<D>(ji, dji, dec, dnd, std::make_integer_sequence<int, NV>{});
-#pragma unroll
-        for (int al = 0; al < D; ++al) {
-          float s = 0.f;
-#pragma unroll
-          for (int a = 1; a < NG; ++a) s += dnd[a][al];
-          xb[0][al] = -s;
-        }
-#pragma unroll
-        for (int k = 1; k <= D; ++k)
-#pragma unroll
-          for (int al = 0; al < D; ++al) xb[k][al] = dnd[k][al];
-#pragma unroll
-        for (int q = 0; q < NE; ++q)
-#pragma unroll
-          for (int al = 0; al < D; ++al) mb[q][al] = dnd[D + 1 + q][al];
-      }
+      if (!ok) err |= DEVERR_DEGENERATE;
     } else if (flags & GF_ELEM) {
       err |= DEVERR_CONN;
     }
+    SymVals<FT::NT> sym;
+    stage_sym<D, FORM>(dslot + lane * PL::DST, sym.s);
+    __syncwarp();  // every lane has read its dA row and its edge nodes
+    copy_dA_async<D, FORM>(p, t + S, lane, dslot);  // the next tile's, while this tile computes
+    cp_async_commit();
+    if (ok) {
+      const float w = (p.coef && e < p.n_elem) ? __ldg(p.coef + e) : 1.f;
+      const float absdet = fabsf(detc);
+      const float sc = w * absdet * (1.f / float(FT::DEN));
+      // 1. the contraction's adjoint; A is homogeneous of degree two in J^{-1}, so
+      // dsc = sum_g s_g H_g is half the sum of J^{-1} times its gradient
+      float dji[NV][D][D];
+      if constexpr (FT::DEG == 1)
+        iso_adjoint_p1<D>(sym.s, ji, dji);
+      else
+        iso_adjoint_p2<D>([&](int k) { return sym.s[k]; }, ji, dji);
+      float dsc = 0.f;
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu)
+#pragma unroll
+          for (int a = 0; a < D; ++a) {
+            dsc = fmaf(ji[k][mu][a], dji[k][mu][a], dsc);
+            dji[k][mu][a] *= sc;
+          }
+      dsc *= 0.5f;
+      // 2. coefficient and centroid determinant
+      dw = dsc * absdet * (1.f / float(FT::DEN));
+      const float ddet = (detc > 0.f ? 1.f : -1.f) * dsc * w * (1.f / float(FT::DEN)) *
+                         (D == 2 ? (1.f / 9.f) : (1.f / 64.f));
+      float dec[D][D];
+#pragma unroll
+      for (int mu = 0; mu < D; ++mu)
+#pragma unroll
+        for (int al = 0; al < D; ++al) dec[mu][al] = ddet * adjc[mu][al];
+      // 3.-4. inverse Jacobians and the centroid term pulled back to the nodes
+      float dnd[NG][D];
+#pragma unroll
+      for (int a = 0; a < NG; ++a)
+#pragma unroll
+        for (int al = 0; al < D; ++al) dnd[a][al] = 0.f;
+      all_vertex_pullback<D>(ji, dji, dec, dnd, std::make_integer_sequence<int, NV>{});
+#pragma unroll
+      for (int al = 0; al < D; ++al) {
+        float s = 0.f;
+#pragma unroll
+        for (int a = 1; a < NG; ++a) s += dnd[a][al];
+        xb[0][al] = -s;
+      }
+#pragma unroll
+      for (int k = 1; k <= D; ++k)
+#pragma unroll
+        for (int al = 0; al < D; ++al) xb[k][al] = dnd[k][al];
+#pragma unroll
+      for (int q = 0; q < NE; ++q)
+#pragma unroll
+        for (int al = 0; al < D; ++al) mb[q][al] = dnd[D + 1 + q][al];
+    }
     if (flags & GF_ELEM) {
       if (p.dcoef) __stcs(p.dcoef + e, dw);
-
       if constexpr (ATOMIC) {
         if (ok && p.dcoords)
 #pragma unroll
@@ -186,8 +211,8 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
       __syncwarp();  // every lane's contributions are staged
       warp_records<D, PL::NC>(xs, p.rec_span, p.rec_dest, rb, rn, ah, p.records, lane);
     }
-    if (dmid) {  // the tile's edge-node gradients through the stage, stored coalesced
-      __syncwarp();  // every lane has read its edge nodes
+    if (dmid) {  // the tile's edge-node gradients through the region, stored coalesced
+      __syncwarp();  // the records are summed
 #pragma unroll
       for (int q = 0; q < NE; ++q)
 #pragma unroll
@@ -195,8 +220,11 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
       __syncwarp();
       tile_store(dmid + t * 32 * (NE * D), ms, cnt * (NE * D), lane);
     }
-    __syncwarp();  // the stages and the dA slot are rewritten next tile
+    __syncwarp();  // the region is rewritten next tile
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = vn[k];
   }
+  cp_async_wait<0>();
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && p.dev_err) atomicOr(p.dev_err, err);
 }

@@ -10,60 +10,30 @@
 //      basis there (small integers, compile time), its adjugate and det, and
 //      J^{-1}_k = adj / det -- the values the projection of Eq. 17 interpolates;
 //   3. |J| = |det J| at the centroid (Eq. 17 keeps |J| outside the integral);
-//   4. G^{(k mu),(l nu)} = w |J| / DEN  sum_a J^{-1}_{mu a,k} J^{-1}_{nu a,l}
-//      over the folded slot pairs (Eq. 18), each entry (without the common
-//      factor w |J| / DEN) added into the accumulators of A as soon as it is
-//      formed (A_ij += K^{ij}_g G_g with K as immediates, g in increasing
-//      order: the sums of the G-first contraction, without holding all of G
-//      in registers), the factor applied once per entry of A, then the same
-//      tile store as the affine kernel (Eq. 19).
+//   4. A_ij = w |J| / DEN sum K^{ij}_{(k mu),(l nu)} J^{-1}_{mu a,k} J^{-1}_{nu a,l}
+//      (Eq. 18) by the structure of K (fem_iso_mat.cuh): P2 tets take 2041
+//      instructions a tile of 32 elements where the sum over the 78 folded
+//      G entries took 3680, outgrew the instruction caches and was bound by
+//      them (64^3 cube: 265 -> 162 us; P1 there 51 us); then the same tile
+//      store as the affine kernel (Eq. 19).
 // The Jacobian steps run in plain FP32: this path serves curved, non-sliver
 // elements; an element with a singular J at a vertex or at the centroid is
 // flagged degenerate and gets A = 0.
 #include "fem_fwd.cuh"
-#include "fem_iso.cuh"
+#include "fem_iso_mat.cuh"
 
 namespace fem {
 
 namespace {
 
-// acc[T] += K'[G][T] * gv over the unique entries T of A (zero terms generate no code).
-template <int D, int FORM, int G, int T>
-__device__ __forceinline__ void kscatter(float* acc, float gv) {
-  using FT = FormTraits<D, FORM>;
-  constexpr int k = Ref<D, FORM>::K.v[G][tri_row(T, FT::N)][tri_col(T, FT::N)];
-  if constexpr (k == 1) {
-    acc[T] += gv;
-  } else if constexpr (k == -1) {
-    acc[T] -= gv;
-  } else if constexpr (k != 0) {
-    acc[T] = fmaf(gv, float(k), acc[T]);
-  }
-}
-
-template <int D, int FORM, int G, int... Ts>
-__device__ __forceinline__ void scatter_g(float* acc, float gv, std::integer_sequence<int, Ts...>) {
-  (kscatter<D, FORM, G, Ts>(acc, gv), ...);
-}
-
-// G_g / scale for the slot pair g = (p, q), p <= q, p = (k mu):
-// sum_a Jinv_{mu a,k} Jinv_{nu a,l}.
-template <int D, int FORM, int G>
-__device__ __forceinline__ void iso_term(const float (&ji)[D + 1][D][D], float* acc) {
-  using FT = FormTraits<D, FORM>;
-  constexpr int pp = tri_row(G, FT::NP), qq = tri_col(G, FT::NP);
-  float s = 0.f;
-#pragma unroll
-  for (int al = 0; al < D; ++al) s = fmaf(ji[pp / D][pp % D][al], ji[qq / D][qq % D][al], s);
-  scatter_g<D, FORM, G>(acc, s, std::make_integer_sequence<int, FT::NT>{});
-}
-
-// acc = scale * sum_g K_g G_g / scale: the common factor scale = w |J| / DEN
-// once per entry of A rather than once per G entry.
-template <int D, int FORM, int... Gs>
-__device__ __forceinline__ void iso_accumulate(const float (&ji)[D + 1][D][D], float scale, float* acc,
-                                               std::integer_sequence<int, Gs...>) {
-  (iso_term<D, FORM, Gs>(ji, acc), ...);
+// acc = the upper triangle of A_e: the sums of fem_iso_mat.cuh times the
+// common factor scale = w |J| / DEN.
+template <int D, int FORM>
+__device__ __forceinline__ void iso_accumulate(const float (&ji)[D + 1][D][D], float scale, float* acc) {
+  if constexpr (FormTraits<D, FORM>::DEG == 1)
+    iso_matrix_p1<D>(ji, acc);
+  else
+    iso_matrix_p2<D>(ji, acc);
 #pragma unroll
   for (int t = 0; t < FormTraits<D, FORM>::NT; ++t) acc[t] *= scale;
 }
@@ -77,10 +47,9 @@ __device__ __forceinline__ void put_all(Sink& sink, const float* acc, std::integ
 // CTA shape: warps never wait for one another, so the CTA size only sets how
 // finely the register file is shared out.  On tets the P1 form runs one-warp
 // CTAs with at least 20 resident per SM, which holds it to 96 registers
-// without spills (21 warps per SM against 16 at 128 registers); the P2 form
-// with at least 16, which holds its 55 accumulators and four inverse
-// Jacobians to 128 registers without spills (16 warps per SM, against 8 at
-// the 245 registers it takes unbounded).
+// without spills (21 warps per SM against 16 at 128 registers; 24 or 32 CTAs
+// spill and gain nothing); the P2 form with at least 16, which holds its 55
+// accumulators and four inverse Jacobians to 128 registers (20 bytes spilled).
 template <int D, int FORM>
 struct IsoShape {
   static constexpr bool tight = (D == 3);
@@ -121,7 +90,7 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
           float acc[FT::NT];
 #pragma unroll
           for (int i = 0; i < FT::NT; ++i) acc[i] = 0.f;
-          if (ok) iso_accumulate<D, FORM>(ji, scale, acc, std::make_integer_sequence<int, FT::NG>{});
+          if (ok) iso_accumulate<D, FORM>(ji, scale, acc);
           put_all<D, FORM>(sink, acc, std::make_integer_sequence<int, FT::NT>{});
         },
         st, nullptr);

@@ -1,7 +1,7 @@
 // fem_iso_adj.cuh -- per-element pieces of the adjoint of the non-affine
-// (quadratic-geometry) forward, Eqs. 16-19, shared by the FP32 adjoint kernel
-// (fem_bwd_iso.cu) and the one whose contraction adjoint runs on the tensor
-// cores (fem_bwd_iso_tc.cu): the slot-pair terms, the pullback of the vertex
+// (quadratic-geometry) forward, Eqs. 16-19: the slot-pair terms of the kernel
+// whose contraction adjoint runs on the tensor cores (fem_bwd_iso_tc.cu) and,
+// shared with the FP32 adjoint kernel (fem_bwd_iso.cu), the pullback of the vertex
 // Jacobians to the geometry nodes, and the 16-byte staging of a tile's edge
 // nodes.
 #pragma once
@@ -34,19 +34,6 @@ __device__ __forceinline__ void iso_adj_apply(float s, const float (&ji)[D + 1][
       dji[kq][mq][a] = fmaf(t, ji[kp][mp][a], dji[kq][mq][a]);
     }
   }
-}
-
-template <int D, int FORM, int G, class Sym>
-__device__ __forceinline__ void iso_adj_term(const Sym& sym, const float (&ji)[D + 1][D][D], float sc,
-                                             float (&dji)[D + 1][D][D], float& dsc) {
-  using FT = FormTraits<D, FORM>;
-  iso_adj_apply<D, FORM, G>(kcol<D, FORM, G>(sym, std::make_integer_sequence<int, FT::NT>{}), ji, sc, dji, dsc);
-}
-
-template <int D, int FORM, class Sym, int... Gs>
-__device__ __forceinline__ void iso_adj_all(const Sym& sym, const float (&ji)[D + 1][D][D], float sc,
-                                            float (&dji)[D + 1][D][D], float& dsc, std::integer_sequence<int, Gs...>) {
-  (iso_adj_term<D, FORM, Gs>(sym, ji, sc, dji, dsc), ...);
 }
 
 // d nd_a[al] += sum_mu dpsi_a/dxi_mu(vertex K) de[mu][al] over the nodes a >= 1.
