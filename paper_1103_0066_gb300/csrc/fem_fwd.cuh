@@ -14,8 +14,9 @@
 // conflict-free row writes), double buffered, and one lane stores the whole
 // tile with a TMA tensor store that undoes the swizzle; without a tensor map
 // (unaligned A) the warp reads the stage back into coalesced 16-byte
-// evict-first stores.  Other shapes use an odd row stride and the coalesced
-// read-out.  Every element is integrated: the final tile is partial (no
+// evict-first stores.  FP32 rows of 36 and 100 floats are staged as they lie in
+// memory and stored by one bulk copy; other shapes use an odd row stride and
+// the coalesced read-out.  Every element is integrated: the final tile is partial (no
 // dropped tail; the tensor store clips rows past the end).
 #pragma once
 #include <cuda_runtime.h>
@@ -66,6 +67,12 @@ struct FwdShape {
   static constexpr int default_warps = tight ? 1 : 4;
 };
 
+// How a warp stores its tile: through a padded stage and 16-byte stores
+// (ST_PLAIN: FP64 matrices, and the fused batch kernels, whose stage the
+// adjoint's dA shares), by one TMA tensor store (ST_TENSOR: 4 x 4 FP32) or by
+// a bulk copy of the stage (ST_BULK: 36 and 100 floats).
+enum : int { ST_PLAIN = 0, ST_TENSOR = 1, ST_BULK = 2 };
+
 // Shared-memory plan of one warp.
 template <int D, int FORM, class CT, class OT>
 struct FwdPlan {
@@ -76,6 +83,18 @@ struct FwdPlan {
   static constexpr size_t per_warp = stage_bytes;
   // TMA store variant (SWZ16 only): two 2 KB stages per warp, 1024-byte aligned
   static constexpr size_t tma_per_warp = 2 * 2048;
+  // Bulk variant: rows of 36 and 100 floats, an odd number of 16-byte chunks,
+  // take 16-byte writes without bank conflicts unpadded, so the stage is the
+  // tile as it lies in memory and one bulk copy stores it.  (144-float rows,
+  // padded by a chunk and copied row by row, and 9-float rows, copied as a
+  // tile, hold more registers and were no faster: step of 61^3 cube elasticity
+  // 309 against 308 us, of 2000 x 2000 x 2 P1 triangles 300 against 279 us.)
+  static constexpr bool BULK = sizeof(OT) == 4 && NN % 4 == 0 && (NN / 4) % 2 == 1;
+  static constexpr size_t bulk_per_warp = size_t(32) * NN * sizeof(OT);
+  static constexpr int plain_store = BULK ? ST_BULK : ST_PLAIN;  // without a tensor map
+  static constexpr size_t stage_of(int st) {
+    return st == ST_TENSOR ? tma_per_warp : st == ST_BULK ? bulk_per_warp : per_warp;
+  }
 };
 
 template <int N, int SST, class OT>
@@ -160,8 +179,15 @@ __device__ __forceinline__ int gather_regs(const CT* coords, int64_t n_vert, int
 
 // A lane's element matrix and the tile's store: fill(sink) hands every unique
 // entry (i <= j) to sink.put<i, j>(value); then the swizzled stage and its TMA
-// tensor store (TMA), else the stage and the warp's coalesced read-out.
-template <int D, int FORM, class CT, class OT, bool TMA, class Fill>
+// tensor store, the stage and its bulk copy, or the stage and the warp's
+// coalesced read-out.
+//
+// The bulk copy takes the read-out off the shared-memory pipe, which bound the
+// P2 tets: scalar writes of a lane's row and four-float reads at an odd stride
+// took 473 wavefronts a tile of 100-float rows, 16-byte writes take 100 and
+// the copy none.  P2 with a P1 coefficient, 72^3 cube, forward 180 -> 160 us;
+// curved P2, 64^3 cube, 162 -> 130 us; 36-float rows gain 0 to 2%.
+template <int D, int FORM, class CT, class OT, int ST, class Fill>
 __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64_t tile, int lane, Fill&& fill,
                                                OT* st, const CUtensorMap* tmap) {
   using FT = FormTraits<D, FORM>;
@@ -171,7 +197,30 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
   const int64_t e0 = tile * 32;
   const int cnt = int(p.n_elem - e0 < 32 ? p.n_elem - e0 : 32);
   OT* dst = p.A + e0 * NN;
-  if constexpr (PL::SWZ16) {
+  constexpr bool TMA = ST == ST_TENSOR;
+  if constexpr (ST == ST_BULK) {
+    float* row = st + lane * NN;
+    // the copy of the last tile has read the stage (waited for before the
+    // contraction, so that its results need not all be held over the wait)
+    if (lane == 0) bulk_wait_read<0>();
+    __syncwarp();
+    RegSink<FT::N, float> rs;
+    fill(rs);
+#pragma unroll
+    for (int q = 0; q < NN / 4; ++q)
+      reinterpret_cast<float4*>(row)[q] = make_float4(rs.a[4 * q], rs.a[4 * q + 1], rs.a[4 * q + 2], rs.a[4 * q + 3]);
+    if (p.vec_store) {
+      fence_proxy_async_smem();  // the rows are visible to the copy
+      __syncwarp();
+      if (lane == 0) {
+        bulk_store_stream(dst, st, uint32_t(cnt) * NN * 4);
+        bulk_commit();
+      }
+      return;
+    }
+    __syncwarp();
+    for (int idx = lane; idx < cnt * NN; idx += 32) __stcs(dst + idx, st[idx]);
+  } else if constexpr (PL::SWZ16) {
     // rows as float4 chunks, chunk index XOR-swizzled with (lane >> 1) & 3
     RegSink<4, float> rs;
     fill(rs);
@@ -246,11 +295,11 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
 }
 
 // Contraction of a lane's folded G with K (immediates), then the tile's store.
-template <int D, int FORM, class CT, class OT, bool TMA = false>
+template <int D, int FORM, class CT, class OT, int ST = ST_PLAIN>
 __device__ __forceinline__ void fwd_contract_store(const FwdParams<CT, OT>& p, int64_t tile, int lane,
                                                    const OT (&Gf)[FormTraits<D, FORM>::NG], OT* st,
                                                    const CUtensorMap* tmap) {
-  fwd_fill_store<D, FORM, CT, OT, TMA>(p, tile, lane, [&](auto& sink) { contract<D, FORM>(Gf, sink); }, st, tmap);
+  fwd_fill_store<D, FORM, CT, OT, ST>(p, tile, lane, [&](auto& sink) { contract<D, FORM>(Gf, sink); }, st, tmap);
 }
 
 // The element's coefficient: one value (per-element coefficient) or the
@@ -273,8 +322,8 @@ __device__ __forceinline__ void load_coef(const float* coef, int64_t e, int64_t 
 }
 
 // Stage 3 for one tile: geometry, contraction, staging and the coalesced store
-// (TMA: the tensor store of the stage through tmap).
-template <int D, int FORM, int JAC, class CT, class OT, bool TMA = false>
+// (ST_TENSOR: the tensor store of the stage through tmap).
+template <int D, int FORM, int JAC, class CT, class OT, int ST = ST_PLAIN>
 __device__ __forceinline__ int fwd_compute_tile(const FwdParams<CT, OT>& p, int64_t tile, int lane, int flags,
                                                 const Coef<FormTraits<D, FORM>::NW>& w, const CT (&X)[D + 1][D],
                                                 OT* st, const CUtensorMap* tmap = nullptr) {
@@ -308,7 +357,7 @@ __device__ __forceinline__ int fwd_compute_tile(const FwdParams<CT, OT>& p, int6
     err |= DEVERR_CONN;
     if (p.det_out) __stcs(p.det_out + tile * 32 + lane, 0.f);
   }
-  fwd_contract_store<D, FORM, CT, OT, TMA>(p, tile, lane, Gf, st, tmap);
+  fwd_contract_store<D, FORM, CT, OT, ST>(p, tile, lane, Gf, st, tmap);
   return err;
 }
 
@@ -323,7 +372,7 @@ __device__ __forceinline__ int fwd_compute_tile(const FwdParams<CT, OT>& p, int6
 // (coordinates, coefficient), then compute and store tile t.  The kernel
 // calls it with the register buffers swapped on alternate steps, so the
 // pipeline rotates without register copies.
-template <int D, int FORM, int JAC, class CT, class OT, bool TMA>
+template <int D, int FORM, int JAC, class CT, class OT, int ST>
 __device__ __forceinline__ void fwd_step(const FwdParams<CT, OT>& p, int64_t t, int64_t S, int lane,
                                          const int (&vnext)[D + 1], int (&vload)[D + 1],
                                          const CT (&Xcur)[D + 1][D], CT (&Xnext)[D + 1][D], int fcur,
@@ -334,20 +383,20 @@ __device__ __forceinline__ void fwd_step(const FwdParams<CT, OT>& p, int64_t t, 
   load_conn<D>(p.conn, (t + 2 * S) * 32 + lane, p.n_elem, p.vec_conn, vload);
   fnext = gather_regs<D>(p.coords, p.n_vert, en, p.n_elem, vnext, Xnext);
   load_coef<D, FORM>(p.coef, en, p.n_elem, p.n_vert, vnext, wnext);
-  err |= fwd_compute_tile<D, FORM, JAC, CT, OT, TMA>(p, t, lane, fcur, wcur, Xcur, st, tmap);
+  err |= fwd_compute_tile<D, FORM, JAC, CT, OT, ST>(p, t, lane, fcur, wcur, Xcur, st, tmap);
 }
 
-template <int D, int FORM, int JAC, class CT, class OT, bool TMA>
+template <int D, int FORM, int JAC, class CT, class OT, int ST>
 __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, CT, OT>::threads, FwdShape<D, FORM, JAC, CT, OT>::min_ctas)
     fem_fwd_kernel(FwdParams<CT, OT> p, const __grid_constant__ CUtensorMap tmap) {
   using PL = FwdPlan<D, FORM, CT, OT>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  // TMA: two 1024-byte-aligned stages per warp (the swizzle follows the shared address)
+  constexpr bool TMA = ST == ST_TENSOR;  // two 1024-byte-aligned stages per warp (the swizzle follows the shared address)
   unsigned char* sbase =
       TMA ? reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023))
           : smem_raw;
-  OT* st = reinterpret_cast<OT*>(sbase + size_t(warp) * (TMA ? PL::tma_per_warp : PL::per_warp));
+  OT* st = reinterpret_cast<OT*>(sbase + size_t(warp) * PL::stage_of(ST));
   OT* st2 = TMA ? st + 2048 / sizeof(OT) : st;
   const int64_t ntiles = (p.n_elem + 31) / 32;
   const int64_t S = int64_t(gridDim.x) * nwarps;
@@ -364,14 +413,12 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, CT, OT>::threads, FwdSh
   load_coef<D, FORM>(p.coef, t * 32 + lane, p.n_elem, p.n_vert, va, wa);
   load_conn<D>(p.conn, (t + S) * 32 + lane, p.n_elem, p.vec_conn, va);
   for (;;) {
-    fwd_step<D, FORM, JAC, CT, OT, TMA>(p, t, S, lane, va, vb, Xa, Xb, fa, wa, fb, wb, st, &tmap, err);
+    fwd_step<D, FORM, JAC, CT, OT, ST>(p, t, S, lane, va, vb, Xa, Xb, fa, wa, fb, wb, st, &tmap, err);
     if ((t += S) >= ntiles) break;
-    fwd_step<D, FORM, JAC, CT, OT, TMA>(p, t, S, lane, vb, va, Xb, Xa, fb, wb, fa, wa, st2, &tmap, err);
+    fwd_step<D, FORM, JAC, CT, OT, ST>(p, t, S, lane, vb, va, Xb, Xa, fb, wb, fa, wa, st2, &tmap, err);
     if ((t += S) >= ntiles) break;
   }
-  if constexpr (TMA) {
-    if (lane == 0) bulk_wait<0>();  // the stages outlive every tensor store that reads them
-  }
+  if constexpr (ST != ST_PLAIN) bulk_wait<0>();  // the stages outlive every copy that reads them
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && p.dev_err) atomicOr(p.dev_err, err);
 }
@@ -392,15 +439,15 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
   p.det_out = L.det_out;
   CUtensorMap tmap{};
   bool tma = false;
-  auto kern = fem_fwd_kernel<D, FORM, JAC, CT, OT, false>;
+  auto kern = fem_fwd_kernel<D, FORM, JAC, CT, OT, PL::plain_store>;
   if constexpr (PL::SWZ16) {
     if (encode_rows16_map(&tmap, L.A, L.n_elem)) {
       tma = true;
-      kern = fem_fwd_kernel<D, FORM, JAC, CT, OT, true>;
+      kern = fem_fwd_kernel<D, FORM, JAC, CT, OT, ST_TENSOR>;
     }
   }
   using SH = FwdShape<D, FORM, JAC, CT, OT>;
-  const size_t per_warp = tma ? PL::tma_per_warp : PL::per_warp;
+  const size_t per_warp = tma ? PL::tma_per_warp : PL::BULK ? PL::bulk_per_warp : PL::per_warp;
   const int want = L.warps > 0 ? L.warps : SH::default_warps;
   const int warps = clamp_warps(want < SH::threads / 32 ? want : SH::threads / 32, per_warp);
   const size_t smem = size_t(warps) * per_warp + (tma ? 1024 : 0);

@@ -14,7 +14,7 @@
 //      (Eq. 18) by the structure of K (fem_iso_mat.cuh): P2 tets take 2041
 //      instructions a tile of 32 elements where the sum over the 78 folded
 //      G entries took 3680, outgrew the instruction caches and was bound by
-//      them (64^3 cube: 265 -> 162 us; P1 there 51 us); then the same tile
+//      them (64^3 cube: 265 -> 162 us, 130 us with the bulk store); then the same tile
 //      store as the affine kernel (Eq. 19).
 // The Jacobian steps run in plain FP32: this path serves curved, non-sliver
 // elements; an element with a singular J at a vertex or at the centroid is
@@ -57,6 +57,20 @@ struct IsoShape {
   static constexpr int min_ctas = tight ? (FORM == LAPLACE_P1_ISO ? 20 : 16) : 1;
 };
 
+// Per warp: [output stage][edge nodes of a tile][its coordinates].  The inputs
+// are copied one tile ahead, except on P2 tets, where the 3.8 KB they take
+// beside the 12.8 KB output stage cost more resident warps than the wait saved
+// (64^3 cube, forward + adjoint 386 against 381 us; P1 tets 173 -> 168 us, P2
+// triangles at 700 x 700 x 2 111 -> 100 us).
+template <int D, int FORM>
+struct IsoFwdPlan {
+  using PL = FwdPlan<D, FORM, float, float>;
+  static constexpr bool ahead = D == 2 || FORM == LAPLACE_P1_ISO;
+  static constexpr size_t stage = PL::stage_of(PL::plain_store);
+  static constexpr size_t mid_bytes = align_up(size_t(32) * (D * D * (D + 1) / 2) * 4, 128);
+  static constexpr size_t per_warp = stage + (ahead ? mid_bytes + 32 * (D + 1) * D * 4 : 0);
+};
+
 template <int D, int FORM>
 __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>::min_ctas)
     fem_fwd_iso_kernel(FwdParams<float, float> p, const float* __restrict__ mid) {
@@ -65,26 +79,73 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
   constexpr int NE = D * (D + 1) / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  float* st = reinterpret_cast<float*>(smem_raw + size_t(warp) * PL::per_warp);
+  using IP = IsoFwdPlan<D, FORM>;
+  unsigned char* wbase = smem_raw + size_t(warp) * IP::per_warp;
+  float* st = reinterpret_cast<float*>(wbase);
+  float* ms = reinterpret_cast<float*>(wbase + IP::stage);                         // [32][NE * D]
+  float* xs = reinterpret_cast<float*>(wbase + IP::stage + IP::mid_bytes) + lane;  // [(D + 1) * D][32]
   const int64_t ntiles = (p.n_elem + 31) / 32;
-  int err = 0;
-  for (int64_t t = int64_t(blockIdx.x) * nwarps + warp; t < ntiles; t += int64_t(gridDim.x) * nwarps) {
+  const int64_t S = int64_t(gridDim.x) * nwarps;
+  int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  if (t >= ntiles) return;  // warp-uniform: the kernel has no CTA-wide barrier
+  int err = 0, fnext = 0;
+  int v[D + 1];
+  load_conn<D>(p.conn, t * 32 + lane, p.n_elem, p.vec_conn, v);
+  // copies tile's edge nodes and, by the vertex ids in v, its coordinates, then
+  // loads the ids of the tile after it; the tile's gather flags
+  auto copy_ahead = [&](int64_t tile) {
+    int flags = 0;
+    if (tile < ntiles) {
+      const int cnt = int(p.n_elem - tile * 32 < 32 ? p.n_elem - tile * 32 : 32);
+      tile_load_async(ms, mid + tile * 32 * (NE * D), cnt * (NE * D), lane);
+      if (lane < cnt) {
+        bool good = true;
+#pragma unroll
+        for (int k = 0; k <= D; ++k) good &= uint32_t(v[k]) < uint32_t(p.n_vert);
+        flags = good ? GF_ELEM | GF_OK : GF_ELEM;
+        if (good)
+#pragma unroll
+          for (int k = 0; k <= D; ++k)
+#pragma unroll
+            for (int a = 0; a < D; ++a) cp_async<4>(xs + (k * D + a) * 32, p.coords + uint32_t(v[k]) * uint64_t(D) + a);
+      }
+    }
+    cp_async_commit();
+    load_conn<D>(p.conn, (tile + S) * 32 + lane, p.n_elem, p.vec_conn, v);
+    return flags;
+  };
+  if constexpr (IP::ahead) fnext = copy_ahead(t);
+  for (; t < ntiles; t += S) {
     const int64_t e = t * 32 + lane;
-    int v[D + 1];
     float X[D + 1][D];
-    load_conn<D>(p.conn, e, p.n_elem, p.vec_conn, v);
-    const int flags = gather_regs<D>(p.coords, p.n_vert, e, p.n_elem, v, X);
+    int flags = fnext;
+    if constexpr (IP::ahead) {
+      cp_async_wait<0>();
+      __syncwarp();  // the tile's edge nodes were copied by other lanes
+#pragma unroll
+      for (int k = 0; k <= D; ++k)
+#pragma unroll
+        for (int a = 0; a < D; ++a) X[k][a] = xs[(k * D + a) * 32];
+    } else {
+      flags = gather_regs<D>(p.coords, p.n_vert, e, p.n_elem, v, X);
+    }
     float ji[D + 1][D][D];
     float scale = 0.f;
     bool ok = false;
     if (flags & GF_OK) {
       const float w = (p.coef && e < p.n_elem) ? __ldg(p.coef + e) : 1.f;
-      ok = iso_geometry<D, FORM>(X, mid + e * (NE * D), w, ji, scale);
+      ok = iso_geometry<D, FORM, IP::ahead>(X, IP::ahead ? ms + lane * (NE * D) : mid + e * (NE * D), w, ji, scale);
       if (!ok) err |= DEVERR_DEGENERATE;
     } else if (flags & GF_ELEM) {
       err |= DEVERR_CONN;
     }
-    fwd_fill_store<D, FORM, float, float, false>(
+    if constexpr (IP::ahead) {
+      __syncwarp();  // every lane has read its edge nodes: the next tile's may arrive
+      fnext = copy_ahead(t + S);
+    } else {
+      load_conn<D>(p.conn, e + S * 32, p.n_elem, p.vec_conn, v);
+    }
+    fwd_fill_store<D, FORM, float, float, PL::plain_store>(
         p, t, lane,
         [&](auto& sink) {
           float acc[FT::NT];
@@ -95,13 +156,14 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
         },
         st, nullptr);
   }
+  cp_async_wait<0>();
+  if constexpr (PL::BULK) bulk_wait<0>();  // the stage outlives every copy that reads it
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && p.dev_err) atomicOr(p.dev_err, err);
 }
 
 template <int D, int FORM>
 cudaError_t launch_iso_t(const FwdLaunch& L, const float* mid) {
-  using PL = FwdPlan<D, FORM, float, float>;
   FwdParams<float, float> p;
   p.conn = L.conn;
   p.coords = static_cast<const float*>(L.coords);
@@ -114,7 +176,7 @@ cudaError_t launch_iso_t(const FwdLaunch& L, const float* mid) {
   p.vec_store = (reinterpret_cast<uintptr_t>(L.A) % 16 == 0);
   auto kern = fem_fwd_iso_kernel<D, FORM>;
   const int warps = IsoShape<D, FORM>::threads / 32;
-  const size_t smem = size_t(warps) * PL::per_warp;
+  const size_t smem = size_t(warps) * IsoFwdPlan<D, FORM>::per_warp;
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);

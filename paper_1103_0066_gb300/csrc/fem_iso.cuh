@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "fem_core.cuh"
+#include "fem_pipe.cuh"
 
 namespace fem {
 
@@ -79,9 +80,10 @@ __device__ __forceinline__ bool all_vertex_jinv(const float (&nd)[n_geo(D)][D], 
 
 // One element's inverse Jacobians at its vertices (ji[k][mu][al] = (J^{-1})_{mu al}
 // at vertex k) and scale = w |det J(centroid)| / DEN, from its vertex
-// coordinates X and its edge nodes m (d(d+1)/2 points, P2 edge order).  False
-// (ji, scale undefined) when J is singular at a vertex or at the centroid.
-template <int D, int FORM>
+// coordinates X and its edge nodes m (d(d+1)/2 points, P2 edge order), in
+// global memory or, staged, in shared memory.  False (ji, scale undefined)
+// when J is singular at a vertex or at the centroid.
+template <int D, int FORM, bool STAGED = false>
 __device__ __forceinline__ bool iso_geometry(const float (&X)[D + 1][D], const float* m, float w,
                                              float (&ji)[D + 1][D][D], float& scale) {
   constexpr int NE = D * (D + 1) / 2;
@@ -93,7 +95,7 @@ __device__ __forceinline__ bool iso_geometry(const float (&X)[D + 1][D], const f
 #pragma unroll
   for (int q = 0; q < NE; ++q)
 #pragma unroll
-    for (int al = 0; al < D; ++al) nd[D + 1 + q][al] = __ldcs(m + q * D + al) - X[0][al];
+    for (int al = 0; al < D; ++al) nd[D + 1 + q][al] = (STAGED ? m[q * D + al] : __ldcs(m + q * D + al)) - X[0][al];
   // J is affine in xi (psi quadratic), so the sum of the vertex Jacobians is
   // (D + 1) J at the centroid
   float ec[D][D], adjc[D][D];
@@ -103,6 +105,26 @@ __device__ __forceinline__ bool iso_geometry(const float (&X)[D + 1][D], const f
   ok &= detc != 0.f;
   scale = w * fabsf(detc) * (1.f / float(FormTraits<D, FORM>::DEN));
   return ok;
+}
+
+// A tile's contiguous run of nf floats between global and shared memory, as
+// 16-byte pieces when both ends allow it (the edge nodes of 32 elements are
+// 2304 bytes on tets, 768 on triangles), else word by word.
+__device__ __forceinline__ void tile_load_async(float* st, const float* g, int nf, int lane) {
+  if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (nf & 3) == 0) {
+    for (int q = lane; q < nf / 4; q += 32) cp_async<16>(st + 4 * q, g + 4 * q);
+  } else {
+    for (int q = lane; q < nf; q += 32) cp_async<4>(st + q, g + q);
+  }
+}
+
+__device__ __forceinline__ void tile_store(float* g, const float* st, int nf, int lane) {
+  if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (nf & 3) == 0) {
+    for (int q = lane; q < nf / 4; q += 32)
+      __stcs(reinterpret_cast<float4*>(g) + q, *reinterpret_cast<const float4*>(st + 4 * q));
+  } else {
+    for (int q = lane; q < nf; q += 32) __stcs(g + q, st[q]);
+  }
 }
 
 }  // namespace fem

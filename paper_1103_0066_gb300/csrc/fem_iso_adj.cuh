@@ -1,9 +1,8 @@
 // fem_iso_adj.cuh -- per-element pieces of the adjoint of the non-affine
 // (quadratic-geometry) forward, Eqs. 16-19: the slot-pair terms of the kernel
 // whose contraction adjoint runs on the tensor cores (fem_bwd_iso_tc.cu) and,
-// shared with the FP32 adjoint kernel (fem_bwd_iso.cu), the pullback of the vertex
-// Jacobians to the geometry nodes, and the 16-byte staging of a tile's edge
-// nodes.
+// shared with the FP32 adjoint kernel (fem_bwd_iso.cu), the pullback of
+// the vertex Jacobians to the geometry nodes.
 #pragma once
 
 #include "fem_bwd.cuh"
@@ -82,26 +81,6 @@ __device__ __forceinline__ void all_vertex_pullback(const float (&ji)[D + 1][D][
                                                     const float (&dec)[D][D], float (&dnd)[n_geo(D)][D],
                                                     std::integer_sequence<int, Ks...>) {
   (vertex_pullback<D, Ks>(ji, dji, dec, dnd), ...);
-}
-
-// A tile's contiguous run of nf floats between global and shared memory, as
-// 16-byte pieces when both ends allow it (the edge nodes of 32 elements are
-// 2304 bytes on tets, 768 on triangles), else word by word.
-__device__ __forceinline__ void tile_load_async(float* st, const float* g, int nf, int lane) {
-  if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (nf & 3) == 0) {
-    for (int q = lane; q < nf / 4; q += 32) cp_async<16>(st + 4 * q, g + 4 * q);
-  } else {
-    for (int q = lane; q < nf; q += 32) cp_async<4>(st + q, g + q);
-  }
-}
-
-__device__ __forceinline__ void tile_store(float* g, const float* st, int nf, int lane) {
-  if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (nf & 3) == 0) {
-    for (int q = lane; q < nf / 4; q += 32)
-      __stcs(reinterpret_cast<float4*>(g) + q, *reinterpret_cast<const float4*>(st + 4 * q));
-  } else {
-    for (int q = lane; q < nf; q += 32) __stcs(g + q, st[q]);
-  }
 }
 
 }  // namespace fem

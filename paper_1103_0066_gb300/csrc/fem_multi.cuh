@@ -68,6 +68,7 @@ __device__ __forceinline__ void fwd_multi_step(const FwdMulti& P, int64_t g, int
                                                const float (&Xcur)[D + 1][D], float (&Xnext)[D + 1][D], int fcur,
                                                const Coef<FormTraits<D, FORM>::NW>& wcur, int& fnext,
                                                Coef<FormTraits<D, FORM>::NW>& wnext, float* st, int& err) {
+  using PL = FwdPlan<D, FORM, float, float>;
   const int m2 = multi_mesh_at(P.tile_begin, P.n, m1, g + 2 * S);
   {
     const FwdParams<float, float>& p = P.p[m2];
@@ -79,7 +80,7 @@ __device__ __forceinline__ void fwd_multi_step(const FwdMulti& P, int64_t g, int
     fnext = gather_regs<D>(p.coords, p.n_vert, en, p.n_elem, vnext, Xnext);
     load_coef<D, FORM>(p.coef, en, p.n_elem, p.n_vert, vnext, wnext);
   }
-  err |= fwd_compute_tile<D, FORM, JAC, float, float, false>(P.p[m0], g - P.tile_begin[m0], lane, fcur, wcur, Xcur,
+  err |= fwd_compute_tile<D, FORM, JAC, float, float, PL::plain_store>(P.p[m0], g - P.tile_begin[m0], lane, fcur, wcur, Xcur,
                                                              st);
   m0 = m1;
   m1 = m2;
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, float, float>::threads,
   using PL = FwdPlan<D, FORM, float, float>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  float* st = reinterpret_cast<float*>(smem_raw + size_t(warp) * PL::per_warp);
+  float* st = reinterpret_cast<float*>(smem_raw + size_t(warp) * PL::stage_of(PL::plain_store));
   const int64_t T = P.tile_begin[P.n];
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t g = int64_t(blockIdx.x) * nwarps + warp;
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, float, float>::threads,
     fwd_multi_step<D, FORM, JAC>(P, g, S, lane, m0, m1, vb, va, Xb, Xa, fb, wb, fa, wa, st, err);
     if ((g += S) >= T) break;
   }
+  if constexpr (PL::BULK) bulk_wait<0>();  // the stage outlives every copy that reads it
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && P.dev_err) atomicOr(P.dev_err, err);
 }
@@ -277,8 +279,9 @@ cudaError_t launch_fwd_multi_t(const FwdMulti& P, cudaStream_t st) {
   const int64_t T = P.tile_begin[P.n];
   if (T == 0) return cudaSuccess;
   auto kern = fem_fwd_multi_kernel<D, FORM, JAC>;
-  const int warps = clamp_warps(SH::default_warps, PL::per_warp);
-  const size_t smem = size_t(warps) * PL::per_warp;
+  constexpr size_t per_warp = PL::stage_of(PL::plain_store);
+  const int warps = clamp_warps(SH::default_warps, per_warp);
+  const size_t smem = size_t(warps) * per_warp;
   cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, T * 32, 0);

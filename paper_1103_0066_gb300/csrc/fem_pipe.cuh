@@ -54,6 +54,14 @@ __device__ __forceinline__ void bulk_store(void* gmem, const void* smem, uint32_
                "r"(bytes)
                : "memory");
 }
+// The same for streamed output (L2 evict-first).
+__device__ __forceinline__ void bulk_store_stream(void* gmem, const void* smem, uint32_t bytes) {
+  asm volatile(
+      "{\n .reg .b64 pol;\n createpolicy.fractional.L2::evict_first.b64 pol, 1.0;\n"
+      " cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, pol;\n}\n" ::"l"(gmem),
+      "r"(smem_u32(smem)), "r"(bytes)
+      : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // Waits until at most N bulk groups of this thread still READ shared memory.
 template <int N>
