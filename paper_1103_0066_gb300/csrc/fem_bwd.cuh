@@ -131,7 +131,28 @@ __device__ __forceinline__ void copy_dA_async(const BwdParams& p, int64_t tile, 
   if (e0 >= p.n_elem) return;
   const int cnt = int(p.n_elem - e0 < 32 ? p.n_elem - e0 : 32);
   const float* src = p.dA + e0 * NN;
-  if constexpr (PL::VEC) {
+  if constexpr (PL::DST == NN && !PL::SWZ) {
+    // unpadded rows (9, 36 or 100 floats): the stage is the tile as it lies in
+    // memory, copied 16 bytes at a time without a division per chunk.  P1
+    // triangles took 9 copies of 4 bytes a lane and 505 instructions a tile in
+    // all: step at 2000 x 2000 x 2 279 -> 257 us with the forward's read-out,
+    // which is of the same kind; curved P2, 64^3 cube, 375 -> 357 us
+    if (p.vec_dA) {
+      constexpr int full = 32 * NN / 4;  // chunks of a full tile
+      float* d = dslot + 4 * lane;
+      const float* s = src + 4 * lane;
+      if (cnt == 32) {
+#pragma unroll
+        for (int q = 0; q < (full + 31) / 32; ++q)
+          if (q < full / 32 || lane < full % 32) cp_async<16>(d + 128 * q, s + 128 * q);
+        return;
+      }
+      const int nq = cnt * NN / 4;
+      for (int q = lane; q < nq; q += 32) cp_async<16>(dslot + 4 * q, src + 4 * q);
+      if (4 * nq + lane < cnt * NN) cp_async<4>(dslot + 4 * nq + lane, src + 4 * nq + lane);
+      return;
+    }
+  } else if constexpr (PL::VEC) {
     if (p.vec_dA) {
       constexpr int Q = NN / 4;
       if constexpr (PL::SWZ) {
@@ -147,16 +168,6 @@ __device__ __forceinline__ void copy_dA_async(const BwdParams& p, int64_t tile, 
           cp_async<16>(dslot + el * 16 + 4 * ((q & 3) ^ ((el >> 1) & 3)), src + 4 * q);
         }
         return;
-      }
-      if constexpr (32 % Q == 0) {
-        if (cnt == 32) {  // full tile: chunk lane + 32 i is chunk lane % Q of row lane / Q + i (32 / Q)
-          constexpr int RPI = 32 / Q;
-          float* d = dslot + (lane / Q) * PL::DST + 4 * (lane % Q);
-          const float* s = src + 4 * lane;
-#pragma unroll
-          for (int i = 0; i < Q; ++i) cp_async<16>(d + i * RPI * PL::DST, s + 128 * i);
-          return;
-        }
       }
       const int nq = cnt * Q;
       for (int q = lane; q < nq; q += 32) {

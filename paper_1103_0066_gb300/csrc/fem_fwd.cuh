@@ -64,7 +64,16 @@ struct FwdShape {
   static constexpr bool tight = tight_ctas() > 0;
   static constexpr int threads = tight ? 32 : 512;
   static constexpr int min_ctas = tight ? tight_ctas() : 1;
-  static constexpr int default_warps = tight ? 1 : 4;
+  // 36 and 100 floats a row (stored by bulk copies): one-warp CTAs
+  static constexpr bool rows36_100 = sizeof(OT) == 4 && (FormTraits<D, FORM>::NN == 36 || FormTraits<D, FORM>::NN == 100);
+  static constexpr int default_warps = tight || rows36_100 ? 1 : 4;
+  // CTAs per SM of the default grid, 0 for as many as are resident.  More than
+  // that lets the hardware hand the last tiles to whichever SM is free, which
+  // evens out the write-bound forms: P2 tets 64^3 112 -> 107 us, P2 with a P1
+  // coefficient 72^3 159 -> 151, 36-float rows at 1023 x 1023 x 2 59.5 -> 56,
+  // elasticity 61^3 140 -> 137.  The 3D P1 forward, bound by latency, and the
+  // adjoints, whose warps start with an exposed copy, lose by it.
+  static constexpr int default_ctas = rows36_100 ? 64 : (D == 3 && FORM == ELASTIC_P1 && sizeof(OT) == 4) ? 8 : 0;
 };
 
 // How a warp stores its tile: through a padded stage and 16-byte stores
@@ -219,6 +228,7 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
       return;
     }
     __syncwarp();
+#pragma unroll 1
     for (int idx = lane; idx < cnt * NN; idx += 32) __stcs(dst + idx, st[idx]);
   } else if constexpr (PL::SWZ16) {
     // rows as float4 chunks, chunk index XOR-swizzled with (lane >> 1) & 3
@@ -271,7 +281,18 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
     fill(sink);
     __syncwarp();
     bool done = false;
-    if constexpr (sizeof(OT) == 4 && NN % 4 == 0) {
+    if constexpr (SST == NN) {  // unpadded rows of odd size: the stage is the tile as it lies in memory
+      constexpr int W = 16 / sizeof(OT);
+      if (p.vec_store) {
+        const int nq = cnt * NN / W;
+#pragma unroll 1
+        for (int q = lane; q < nq; q += 32)
+          __stcs(reinterpret_cast<int4*>(dst) + q, reinterpret_cast<const int4*>(st)[q]);
+#pragma unroll 1
+        for (int idx = W * nq + lane; idx < cnt * NN; idx += 32) __stcs(dst + idx, st[idx]);
+        done = true;
+      }
+    } else if constexpr (sizeof(OT) == 4 && NN % 4 == 0) {
       if (p.vec_store) {
         const int nq = cnt * (NN / 4);
         for (int q = lane; q < nq; q += 32) {
@@ -285,6 +306,7 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
     }
     if (!done) {
       const int nw = cnt * NN;
+#pragma unroll 1
       for (int idx = lane; idx < nw; idx += 32) {
         const int el = idx / NN;
         __stcs(dst + idx, st[el * SST + (idx - el * NN)]);
@@ -453,7 +475,8 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
   const size_t smem = size_t(warps) * per_warp + (tma ? 1024 : 0);
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
-  const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);
+  const int ctas = L.ctas_per_sm > 0 || L.warps > 0 ? L.ctas_per_sm : SH::default_ctas;
+  const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, ctas);
   kern<<<grid, warps * 32, smem, L.stream>>>(p, tmap);
   return cudaGetLastError();
 }
