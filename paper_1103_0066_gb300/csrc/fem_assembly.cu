@@ -589,6 +589,11 @@ struct AsmP2Layout {
   int32_t* eoff;   // [V + 1]
   int32_t* dofs;   // [E][n]
   int32_t* n_rows; // one word: V + n_edges
+  // the rows' incidences in chunks of four: row r holds chunks [choff[r], choff[r+1])
+  int32_t* choff;   // [rows + 1]
+  int4* slot4;      // offsets of the element rows in A, (e * n + i) * n; -1 in the padding
+  uint32_t* pos4;   // [chunk][n]: byte u = the column position of the element's unknown j for incidence u
+  int64_t chunk_cap;
   int64_t rows_cap;
   size_t bytes;
 };
@@ -626,6 +631,15 @@ AsmP2Layout asm_p2_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
   const size_t o_eoff = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_dofs = take(sizeof(int32_t) * size_t(n_elem * n));
   const size_t o_flag = take(sizeof(int32_t) * 8);
+  // 2.9 chunks per tet on a cube; a mesh that needs more room than this (many
+  // unknowns with few elements each) reads the incidences one by one instead
+  L.chunk_cap = n_elem * 9 / 2 + n_vert + 1024;
+  const size_t o_choff = take(sizeof(int32_t) * size_t(rows_cap + 1));
+  const size_t o_slot4 = take(sizeof(int4) * size_t(L.chunk_cap));
+  const size_t o_pos4 = take(sizeof(uint32_t) * size_t(L.chunk_cap * n));
+  L.choff = reinterpret_cast<int32_t*>(b + o_choff);
+  L.slot4 = reinterpret_cast<int4*>(b + o_slot4);
+  L.pos4 = reinterpret_cast<uint32_t*>(b + o_pos4);
   L.eoff = reinterpret_cast<int32_t*>(b + o_eoff);
   L.dofs = reinterpret_cast<int32_t*>(b + o_dofs);
   L.g1.flag = reinterpret_cast<int32_t*>(b + o_flag);
@@ -704,6 +718,36 @@ __global__ void store_rows_kernel(const int32_t* __restrict__ eoff, int64_t n_ve
   if (blockIdx.x == 0 && threadIdx.x == 0) *n_rows = int32_t(n_vert + eoff[n_vert]);
 }
 
+// Chunks of four incidences per row.
+__global__ void chunk_count_kernel(const int32_t* __restrict__ inc_off, int64_t n_rows, int32_t* cnt) {
+  for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < n_rows; r += int64_t(gridDim.x) * blockDim.x)
+    cnt[r] = (inc_off[r + 1] - inc_off[r] + 3) / 4;
+}
+
+template <int NB>
+__global__ void chunk_fill_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ choff,
+                                  int64_t n_rows, int64_t cap, int4* __restrict__ slot4, uint32_t* __restrict__ pos4) {
+  if (choff[n_rows] > cap) return;  // no room: the rows are read one incidence at a time
+  for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < n_rows; r += int64_t(gridDim.x) * blockDim.x) {
+    const int32_t t0 = inc_off[r], n = inc_off[r + 1] - t0;
+    for (int k = 0; k < n; k += 4) {
+      const int64_t c = choff[r] + k / 4;
+      int32_t s[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] = k + u < n ? inc[t0 + k + u] * NB : -1;  // fits: n_elem * NB^2 does
+      slot4[c] = make_int4(s[0], s[1], s[2], s[3]);
+      for (int j = 0; j < NB; ++j) {
+        uint32_t w = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u < n) w |= uint32_t(colpos[(int64_t(t0) + k + u) * NB + j]) << (8 * u);
+        pos4[c * NB + j] = w;
+      }
+    }
+  }
+}
+
 // The P2 build: vertex-graph pattern, edge numbers, element unknowns, then
 // the unknowns' pattern.  Returns the unknown count and the flags (host).
 template <int NV>
@@ -761,6 +805,13 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
   if (e == cudaSuccess && R > 0) {
     row_pattern_kernel<NB, true><<<gr, kPatWarps * 32, 0, st>>>(L.dofs, G2.inc_off, G2.inc, R, G2.cursor,
                                                                  G2.row_ptr, G2.col_idx, G2.colpos, G2.flag);
+    chunk_count_kernel<<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, R, G2.cursor);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = launch_exclusive_scan(G2.cursor, R, G2.partials, L.choff, st);
+  if (e == cudaSuccess && R > 0) {
+    chunk_fill_kernel<NB><<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, G2.inc, G2.colpos, L.choff, R, L.chunk_cap,
+                                                           L.slot4, L.pos4);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(nnz_host, G2.row_ptr + R, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
@@ -773,73 +824,149 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
 // takes its own row, which accumulates in shared memory (at most kMaxCols
 // columns).  For each incidence (e, i) of the row, in increasing element
 // order, lane j of the group adds A_e[i][j] at the column position of the
-// element's unknown j (distinct within an element); the group then stores the
-// row, zeroing the buffer behind it.  Each entry is the sum of its
-// contributions in element order.  The incidences' slots, positions and
-// element rows are loaded NB incidences at a time before their additions.
-constexpr int kRowWarps = 8;
+// element's unknown j (distinct within an element); the warp then stores the
+// rows, which lie side by side, and zeroes the buffers behind them.  Each
+// entry is the sum of its contributions in element order.
+//
+// The incidences come in chunks of four: a lane takes their four slots with one
+// 16-byte load and their four positions with one word, where a slot passed
+// between lanes and a byte per incidence took two shuffles or loads for every
+// addition, on the pipe that the additions use (shared-memory and load pipe
+// 76% busy).  The next two chunks, of this row group or the next, are loaded
+// under the additions.  61^3 cube: 312 -> 281 us; bound by instruction issue
+// (68% active) and that pipe (70%), two accesses an addition, 2.6 wavefronts
+// each over the random columns of three rows.  48 registers: five warps of
+// these buffers per SM quarter and more (40 registers spill: 330 us, 63
+// registers 309 us, without the loads ahead 314 us).
+// A warp with a row of more than kRowCols columns, or a mesh without room for
+// the chunks, takes its rows one after another, an incidence at a time.
+constexpr int kRowWarps = 4;
+constexpr int kRowCols = 160;
+constexpr int kRowStride = kRowCols + 11;  // the rows of a warp start 11 banks apart
+static_assert(3 * kRowStride >= kMaxCols, "one row of any length in the buffers of three");
 
 template <int NB>
-__global__ void __launch_bounds__(kRowWarps * 32)
+__global__ void __launch_bounds__(kRowWarps * 32, 10)
     assemble_rows_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
                          const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                         const float* __restrict__ A, const int32_t* __restrict__ n_rows_dev,
-                         float* __restrict__ val) {
+                         const int32_t* __restrict__ choff, const int4* __restrict__ slot4,
+                         const uint32_t* __restrict__ pos4, int64_t chunk_cap, const float* __restrict__ A,
+                         const int32_t* __restrict__ n_rows_dev, float* __restrict__ val) {
   constexpr int G = 32 / NB;  // rows per warp
-  // row buffers 267 floats apart: the three rows of a warp start 11 banks apart
-  constexpr int kRowStride = kMaxCols + 12;
-  __shared__ float acc_s[kRowWarps][G][kRowStride];
+  constexpr int kWarpRows = G * kRowStride + 1;  // and a word for the lanes without a row
+  __shared__ float acc_s[kRowWarps][kWarpRows];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane / NB, j = lane - g * NB;
-  const bool member = g < G;
-  float* acc = acc_s[warp][member ? g : 0];
+  float* rows = acc_s[warp];
+  float* acc = rows + g * kRowStride;
   // the row buffers are zero at the start of every row: zeroed once here, and
   // each column zeroed again as it is stored
-  for (int c = lane; c < G * kRowStride; c += 32) (&acc_s[warp][0][0])[c] = 0.f;
+  for (int c = lane; c < kWarpRows; c += 32) rows[c] = 0.f;
+  __syncwarp();
+  const float* Aj = A + j;
   const int64_t n_rows = *n_rows_dev;
-  for (int64_t r0 = (int64_t(blockIdx.x) * kRowWarps + warp) * G; r0 < n_rows;
-       r0 += int64_t(gridDim.x) * kRowWarps * G) {
-    const int64_t r = r0 + g;
-    const bool live = member && r < n_rows;
-    const int32_t rp = live ? row_ptr[r] : 0;
-    const int len = live ? row_ptr[r + 1] - rp : 0;
-    const int32_t tb = live ? inc_off[r] : 0;
-    const int n_inc = live ? inc_off[r + 1] - tb : 0;
-    __syncwarp();
-    const int steps = __reduce_max_sync(0xffffffffu, n_inc);
-    // NB incidences at a time: lane j of the group loads incidence k0 + j's
-    // element slot and every incidence's column position j, then (after a
-    // shuffle of the slots) the NB element rows, then the additions in order
-    for (int k0 = 0; k0 < steps; k0 += NB) {
-      const int32_t my_sl = (k0 + j < n_inc) ? __ldg(inc + tb + k0 + j) : 0;
-      int pos[NB];
+  const bool chunked = choff[n_rows] <= chunk_cap;
+  const int64_t S = int64_t(gridDim.x) * kRowWarps * G;
+  int64_t r0 = (int64_t(blockIdx.x) * kRowWarps + warp) * G;
+  if (r0 >= n_rows) return;  // warp-uniform: no CTA-wide barrier
+  // chunks [c0, c0 + nch) of the lane's row, its first value, the values of the warp's rows
+  struct Rows {
+    int32_t c0, nch, rp, total;
+  };
+  auto load_rows = [&](int64_t q0) {
+    Rows m{0, 0, 0, 0};
+    if (q0 >= n_rows) return m;
+    const int64_t r = q0 + g;
+    const bool live = g < G && r < n_rows;
+    m.c0 = live ? __ldg(choff + r) : 0;
+    m.nch = live ? __ldg(choff + r + 1) - m.c0 : 0;
+    m.rp = __ldg(row_ptr + (r < n_rows ? r : n_rows));
+    m.total = __ldg(row_ptr + (q0 + G < n_rows ? q0 + G : n_rows));  // minus the first row's rp
+    return m;
+  };
+  int32_t sn[8];  // slots and positions of the next two chunks
+  uint32_t pn[2];
+  auto load_chunks = [&](const Rows& m, int k) {
 #pragma unroll
-      for (int u = 0; u < NB; ++u) pos[u] = (k0 + u < n_inc) ? __ldg(colpos + (int64_t(tb) + k0 + u) * NB + j) : 0;
-      float a[NB];
+    for (int h = 0; h < 2; ++h) {
+      const bool on = k + h < m.nch;
+      const int64_t c = int64_t(m.c0) + k + h;
+      const int4 q = on ? __ldg(slot4 + c) : make_int4(-1, -1, -1, -1);
+      sn[4 * h] = q.x, sn[4 * h + 1] = q.y, sn[4 * h + 2] = q.z, sn[4 * h + 3] = q.w;
+      pn[h] = on ? __ldg(pos4 + c * NB + j) : 0u;
+    }
+  };
+  Rows m = load_rows(r0);
+  if (chunked) load_chunks(m, 0);
+  for (; r0 < n_rows; r0 += S) {
+    const Rows mn = load_rows(r0 + S);
+    const int32_t rp0 = __shfl_sync(0xffffffffu, m.rp, 0);
+    int32_t first[G + 1];  // of each row, within the warp's run of values
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        const int32_t sl = __shfl_sync(0xffffffffu, my_sl, (member ? g * NB : 0) + u);
-        // slot sl = e * NB + i: row i of A_e starts at e * NB * NB + i * NB = sl * NB
-        a[u] = (k0 + u < n_inc) ? __ldg(A + int64_t(sl) * NB + j) : 0.f;
+    for (int h = 0; h < G; ++h) first[h] = __shfl_sync(0xffffffffu, m.rp, h * NB) - rp0;
+    first[G] = m.total - rp0;
+    bool fast = chunked;
+#pragma unroll
+    for (int h = 0; h < G; ++h) fast &= first[h + 1] - first[h] <= kRowCols;
+    if (fast) {
+      const int steps = __reduce_max_sync(0xffffffffu, m.nch);
+      if (steps == 0) load_chunks(mn, 0);
+      // two chunks at a time: their eight element rows, the next two chunks'
+      // slots and positions, then the additions in order
+      for (int k = 0; k < steps; k += 2) {
+        const uint32_t p[2] = {pn[0], pn[1]};
+        float a[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u] = sn[u] >= 0 ? __ldg(Aj + sn[u]) : 0.f;
+        if (k + 2 < steps)
+          load_chunks(m, k + 2);
+        else
+          load_chunks(mn, 0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (k + h >= steps) break;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            // the padding adds a zero to column 0 (the lanes of a group alike)
+            acc[(p[h] >> (8 * u)) & 0xFFu] += a[4 * h + u];
+            __syncwarp();
+          }
+        }
       }
+      for (int x = lane; x < first[G]; x += 32) {
+        int at = x;
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        if (k0 + u < n_inc) acc[pos[u]] += a[u];
+        for (int h = 1; h < G; ++h)
+          if (x >= first[h]) at = x - first[h] + h * kRowStride;
+        __stcs(val + int64_t(rp0) + x, rows[at]);
+        rows[at] = 0.f;
+      }
+      __syncwarp();  // the row buffers are refilled for the next rows
+    } else {
+      if (chunked) load_chunks(mn, 0);
+      for (int h = 0; h < G && r0 + h < n_rows; ++h) {
+        const int32_t tb = __ldg(inc_off + r0 + h), te = __ldg(inc_off + r0 + h + 1);
+        for (int32_t t = tb; t < te; ++t) {
+          if (lane < NB)
+            rows[__ldg(colpos + int64_t(t) * NB + lane)] += __ldg(A + int64_t(__ldg(inc + t)) * NB + lane);
+          __syncwarp();
+        }
+        const int32_t rp = __ldg(row_ptr + r0 + h), len = __ldg(row_ptr + r0 + h + 1) - rp;
+        for (int x = lane; x < len; x += 32) {
+          __stcs(val + int64_t(rp) + x, rows[x]);
+          rows[x] = 0.f;
+        }
         __syncwarp();
       }
     }
-    for (int c = j; c < len; c += NB) {
-      __stcs(val + rp + c, acc[c]);
-      acc[c] = 0.f;
-    }
-    __syncwarp();  // the row buffers are refilled for the next rows
+    m = mn;
   }
 }
 
 template <int NB>
 cudaError_t launch_p2_assemble(const AsmP2Layout& L, const float* A, float* val, cudaStream_t st) {
   assemble_rows_kernel<NB><<<grid_of(L.rows_cap, kRowWarps * (32 / NB)), kRowWarps * 32, 0, st>>>(
-      L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, A, L.n_rows, val);
+      L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, L.choff, L.slot4, L.pos4, L.chunk_cap, A, L.n_rows, val);
   return cudaGetLastError();
 }
 

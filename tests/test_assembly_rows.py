@@ -11,7 +11,7 @@ import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
-LP1, EP1 = 0, 2
+LP1, LP2, EP1 = 0, 1, 2
 DEV = "cuda:0"
 
 
@@ -73,3 +73,40 @@ def test_row_paths_bitwise(gfem, dim, form, shape, offset):
     else:
         np.add.at(want, inv, blocks)
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("shape", ["long", "single", "wheels"])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_p2_row_paths_bitwise(gfem, dim, shape, offset):
+    """Vertex and edge unknowns: a vertex with more columns than a row buffer
+    of the fast path holds beside short rows, elements that share nothing (one
+    incidence per unknown: more chunks than their room), and closed fans."""
+    nv, nb = dim + 1, (dim + 1) * (dim + 2) // 2
+    if shape == "long":  # 60 triangles: 181 columns (45 tets around an edge: 231)
+        conn = _wheel(dim, 60 if dim == 2 else 45, 0)[0] + [list(range(200, 200 + nv))]
+        V = 210
+    elif shape == "single":
+        conn, V = [list(range(nv * e, nv * e + nv)) for e in range(2000)], nv * 2000 + 1
+    else:
+        conn, V = [el for k in range(7) for el in _wheel(dim, 5 + k, 16 * k)[0]], 16 * 8
+    rng = np.random.default_rng(7)
+    conn = np.ascontiguousarray(np.array(conn, np.int32)[rng.permutation(len(conn))])
+    E = len(conn)
+    A = rng.standard_normal((E, nb, nb)).astype(np.float32)
+    buf = torch.zeros(offset + A.size, device=DEV)
+    buf[offset:] = torch.from_numpy(A.ravel()).to(DEV)
+    asm = gfem.Assembly(torch.zeros((V, dim), device=DEV), torch.from_numpy(conn).to(DEV), LP2)
+    got = [asm.assemble(buf[offset:].view(E, nb, nb)).cpu().numpy() for _ in range(2)]
+    pairs = [(a, b) for a in range(nv) for b in range(a + 1, nv)]
+    lo = np.stack([np.minimum(conn[:, a], conn[:, b]) for a, b in pairs], 1).astype(np.int64)
+    hi = np.stack([np.maximum(conn[:, a], conn[:, b]) for a, b in pairs], 1)
+    _, edge = np.unique(lo * V + hi, return_inverse=True)
+    dofs = np.concatenate([conn, V + edge.reshape(E, -1)], 1)
+    assert np.array_equal(asm.dofs.cpu().numpy(), dofs)
+    key = np.repeat(dofs, nb, axis=1).ravel().astype(np.int64) * asm.n_rows + np.tile(dofs, (1, nb)).ravel()
+    uk, inv = np.unique(key, return_inverse=True)
+    assert asm.nnz == len(uk) and np.array_equal(asm.col_idx.cpu().numpy(), uk % asm.n_rows)
+    want = np.zeros(len(uk), np.float32)
+    np.add.at(want, inv, A.ravel())
+    assert np.array_equal(got[0], want) and np.array_equal(got[1], want)
