@@ -16,6 +16,8 @@ Quick use::
 """
 from __future__ import annotations
 
+import functools
+
 import torch
 
 from . import _native as nat
@@ -40,6 +42,7 @@ def form_info(form: int, dim: int):
     return nat.fem_form_info(form, dim)
 
 
+@functools.lru_cache(maxsize=None)
 def form_shape(form: int, dim: int):
     """(rows, cols) of the form's element blocks: (n, n), or (d+1, d * nbv) for
     the coupling forms DIV_P1P1 / DIV_P2P1."""
@@ -55,7 +58,15 @@ def reference_tensor(form: int, dim: int):
     return K, den
 
 
+# The current stream's handle without the Stream object that
+# torch.cuda.current_stream() builds (0.4 us against 3.3 us, of the 17 us that a
+# small forward took from Python).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
+    if stream is None and _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
     s = stream if stream is not None else torch.cuda.current_stream()
     return int(s.cuda_stream)
 
@@ -479,15 +490,14 @@ class _IntegrateFn(torch.autograd.Function):
         det = torch.empty(mesh.conn.shape[0], dtype=torch.float32, device=coords.device) if keep else None
         A = integrate_fwd(coords, mesh.conn, form, coef, jac=jac, contract=contract, det_out=det)
         ctx.det = det
-        ctx.save_for_backward(coords, coef if coef is not None else torch.empty(0))
+        ctx.save_for_backward(coords, *(() if coef is None else (coef,)))
         ctx.mesh, ctx.form, ctx.jac, ctx.reduce = mesh, form, jac, reduce
         ctx.has_coef = coef is not None
         return A
 
     @staticmethod
     def backward(ctx, dA):
-        coords, coef = ctx.saved_tensors
-        coef = coef if ctx.has_coef else None
+        coords, coef = ctx.saved_tensors if ctx.has_coef else (*ctx.saved_tensors, None)
         need_x = ctx.needs_input_grad[0]
         need_w = ctx.has_coef and ctx.needs_input_grad[1]
         w1 = ctx.form in (LAPLACE_P1_W1, LAPLACE_P2_W1)
@@ -503,14 +513,13 @@ class _IntegrateIsoFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, coords, mid, coef, mesh, form, reduce):
         A = integrate_fwd_iso(coords, mesh.conn, mid, form, coef)
-        ctx.save_for_backward(coords, mid, coef if coef is not None else torch.empty(0))
+        ctx.save_for_backward(coords, mid, *(() if coef is None else (coef,)))
         ctx.mesh, ctx.form, ctx.reduce, ctx.has_coef = mesh, form, reduce, coef is not None
         return A
 
     @staticmethod
     def backward(ctx, dA):
-        coords, mid, coef = ctx.saved_tensors
-        coef = coef if ctx.has_coef else None
+        coords, mid, coef = ctx.saved_tensors if ctx.has_coef else (*ctx.saved_tensors, None)
         need_x, need_m = ctx.needs_input_grad[0], ctx.needs_input_grad[1]
         need_w = ctx.has_coef and ctx.needs_input_grad[2]
         ws = ctx.mesh.workspace(ctx.form) if (need_x and ctx.reduce != REDUCE_ATOMIC) else None

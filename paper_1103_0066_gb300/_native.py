@@ -71,6 +71,8 @@ _lib = None
 def load():
     """Loads the library (it must have been built, e.g. by __graft_entry__.build())."""
     global _lib
+    if _lib is not None:  # set once, under the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
