@@ -134,6 +134,14 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
     __syncwarp();  // every lane has read its dA row and its edge nodes
     copy_dA_async<D, FORM>(p, t + S, lane, dslot);  // the next tile's, while this tile computes
     cp_async_commit();
+    // the next tile's edge nodes wait for the region, but can be in L2 by then
+    // (P1 tets, 64^3 cube, forward + adjoint 167 -> 159 us; P2, bound by issue,
+    // loses: 356 against 360 us)
+    if (D == 3 && FT::DEG == 1 && t + S < ntiles) {
+      const int left = int(p.n_elem - (t + S) * 32 < 32 ? p.n_elem - (t + S) * 32 : 32);
+      prefetch_l2(mid + (t + S) * 32 * (NE * D), left * NE * D * 4, lane);
+      if (rec) prefetch_l2(p.rank + (t + S) * 32, 128, lane);
+    }
     if (ok) {
       const float w = (p.coef && e < p.n_elem) ? __ldg(p.coef + e) : 1.f;
       const float absdet = fabsf(detc);

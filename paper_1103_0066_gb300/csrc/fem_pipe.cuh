@@ -42,6 +42,12 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Fetches into L2 the 128-byte lines of [p, p + bytes), one a lane (bytes <= 4096).
+__device__ __forceinline__ void prefetch_l2(const void* p, int bytes, int lane) {
+  if (lane * 128 < bytes)
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(static_cast<const char*>(p) + lane * 128) : "memory");
+}
+
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy (TMA) reads of the same memory.
 __device__ __forceinline__ void fence_proxy_async_smem() {
