@@ -301,7 +301,7 @@ template <int NV, int B>
 __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ctas)
     assemble_blocks_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
                            const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                           const int32_t* __restrict__ blk_off, const int2* __restrict__ slots, int64_t slot_cap,
+                           const int32_t* blk_off, const int2* __restrict__ slots, int64_t slot_cap,
                            const float* __restrict__ A, int64_t n_vert, float* __restrict__ val, int vec_A) {
   using BP = BlockPlan<B>;
   constexpr int BB = B * B, G = block_rows(B), N = NV * B, U = BP::batch;
@@ -316,10 +316,12 @@ __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ct
   // offset of the component's row and columns in A_e, without the element slot
   const float* Aq = A + (B == 1 ? 0 : (q / B) * NV * N + (q % B) * NV);
   const int64_t nblk = (n_vert + G - 1) / G;
+  int64_t b = int64_t(blockIdx.x) * BP::warps + warp;
+  grid_wait(b, blk_off);
   const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
   // the sums are zero at the start of every block: zeroed here, and again as they are read out
   for (int c = 0; c <= kFastCols; ++c) *reinterpret_cast<float*>(mine + c * 128) = 0.f;
-  for (int64_t b = int64_t(blockIdx.x) * BP::warps + warp; b < nblk; b += int64_t(gridDim.x) * BP::warps) {
+  for (; b < nblk; b += int64_t(gridDim.x) * BP::warps) {
     const int64_t r0 = b * G;
     const int nr = int(n_vert - r0 < G ? n_vert - r0 : G);
     const int32_t s0 = __ldg(blk_off + b), steps = __ldg(blk_off + b + 1) - s0;
@@ -564,9 +566,8 @@ cudaError_t launch_assemble_t(const AsmLayout& L, const float* A, int64_t n_vert
   if (e != cudaSuccess) return e;
   const int64_t nblk = (n_vert + block_rows(B) - 1) / block_rows(B);
   const unsigned g = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, nblk * 32, 0);
-  kern<<<g, warps * 32, smem, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off, L.slots, L.slot_cap, A, n_vert,
-                                    val, int(reinterpret_cast<uintptr_t>(A) % 16 == 0));
-  return cudaGetLastError();
+  return launch_chained(kern, g, unsigned(warps * 32), smem, st, L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off,
+                        L.slots, L.slot_cap, A, n_vert, val, int(reinterpret_cast<uintptr_t>(A) % 16 == 0));
 }
 
 // ------------------------------------------------------------------ P2 unknowns (vertices, then edges)
@@ -851,7 +852,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
                          const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
                          const int32_t* __restrict__ choff, const int4* __restrict__ slot4,
                          const uint32_t* __restrict__ pos4, int64_t chunk_cap, const float* __restrict__ A,
-                         const int32_t* __restrict__ n_rows_dev, float* __restrict__ val) {
+                         const int32_t* n_rows_dev, float* __restrict__ val) {
   constexpr int G = 32 / NB;  // rows per warp
   constexpr int kWarpRows = G * kRowStride + 1;  // and a word for the lanes without a row
   __shared__ float acc_s[kRowWarps][kWarpRows];
@@ -864,10 +865,11 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
   for (int c = lane; c < kWarpRows; c += 32) rows[c] = 0.f;
   __syncwarp();
   const float* Aj = A + j;
+  int64_t r0 = (int64_t(blockIdx.x) * kRowWarps + warp) * G;
+  grid_wait(r0, n_rows_dev);
   const int64_t n_rows = *n_rows_dev;
   const bool chunked = choff[n_rows] <= chunk_cap;
   const int64_t S = int64_t(gridDim.x) * kRowWarps * G;
-  int64_t r0 = (int64_t(blockIdx.x) * kRowWarps + warp) * G;
   if (r0 >= n_rows) return;  // warp-uniform: no CTA-wide barrier
   // chunks [c0, c0 + nch) of the lane's row, its first value, the values of the warp's rows
   struct Rows {
@@ -965,9 +967,9 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
 
 template <int NB>
 cudaError_t launch_p2_assemble(const AsmP2Layout& L, const float* A, float* val, cudaStream_t st) {
-  assemble_rows_kernel<NB><<<grid_of(L.rows_cap, kRowWarps * (32 / NB)), kRowWarps * 32, 0, st>>>(
-      L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, L.choff, L.slot4, L.pos4, L.chunk_cap, A, L.n_rows, val);
-  return cudaGetLastError();
+  return launch_chained(assemble_rows_kernel<NB>, grid_of(L.rows_cap, kRowWarps * (32 / NB)), kRowWarps * 32, 0, st,
+                        L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, L.choff, L.slot4, L.pos4, L.chunk_cap, A,
+                        L.n_rows, val);
 }
 
 }  // namespace

@@ -526,6 +526,7 @@ __global__ void __launch_bounds__(BwdShape<D, FORM, JAC>::threads, BwdShape<D, F
   const int64_t ntiles = (p.n_elem + 31) / 32;
   const int64_t S = int64_t(gridDim.x) * nwarps;  // warp-tile stride
   int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(t);
   if (t >= ntiles) return;  // warp-uniform: the kernel has no CTA-wide barrier
   int err = 0;
   int v1[D + 1], v2[D + 1], vc[D + 1];
@@ -626,8 +627,7 @@ cudaError_t launch_bwd_t(const BwdLaunch& L) {
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);
-  kern<<<grid, warps * 32, smem, L.stream>>>(p);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p);
 }
 
 cudaError_t launch_bwd_elem_w1(const BwdLaunch& L);  // fem_bwd_w1.cu

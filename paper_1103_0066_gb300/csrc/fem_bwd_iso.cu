@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(IsoBwdShape<D, FORM>::threads, IsoBwdShape<D, 
   int err = 0;
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(t);
   if (t >= ntiles) return;  // warp-uniform: the kernel has no CTA-wide barrier
   int v[NV], vn[NV];
   copy_dA_async<D, FORM>(p, t, lane, dslot);
@@ -262,8 +263,7 @@ cudaError_t launch_bwd_iso_t(const BwdLaunch& L, const float* mid, float* dmid) 
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);
-  kern<<<grid, warps * 32, smem, L.stream>>>(p, mid, dmid);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p, mid, dmid);
 }
 
 template <int D, int FORM>

@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, CT, OT>::threads, FwdSh
   const int64_t ntiles = (p.n_elem + 31) / 32;
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(t);
   if (t >= ntiles) return;  // warp-uniform
   int err = 0;
   int va[D + 1], vb[D + 1];
@@ -477,8 +478,7 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
   if (st != cudaSuccess) return st;
   const int ctas = L.ctas_per_sm > 0 || L.warps > 0 ? L.ctas_per_sm : SH::default_ctas;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, ctas);
-  kern<<<grid, warps * 32, smem, L.stream>>>(p, tmap);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p, tmap);
 }
 
 // Dispatch one (D, FORM) over the precision combinations the ABI accepts.

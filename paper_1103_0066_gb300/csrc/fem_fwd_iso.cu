@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
   const int64_t ntiles = (p.n_elem + 31) / 32;
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t t = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(t);
   if (t >= ntiles) return;  // warp-uniform: the kernel has no CTA-wide barrier
   int err = 0, fnext = 0;
   int v[D + 1];
@@ -180,8 +181,7 @@ cudaError_t launch_iso_t(const FwdLaunch& L, const float* mid) {
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);
-  kern<<<grid, warps * 32, smem, L.stream>>>(p, mid);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p, mid);
 }
 
 }  // namespace

@@ -394,9 +394,10 @@ __device__ __forceinline__ void reduce_gather(const int32_t* __restrict__ voff, 
 }
 
 template <int D, int NC>
-__global__ void vertex_reduce_kernel(const int32_t* __restrict__ voff, const int32_t* __restrict__ vrec,
-                                     const int32_t* __restrict__ mode, const float* __restrict__ records,
+__global__ void vertex_reduce_kernel(const int32_t* voff, const int32_t* __restrict__ vrec,
+                                     const int32_t* mode, const float* __restrict__ records,
                                      int64_t n_vert, float* __restrict__ dcoords, float* __restrict__ dcoef) {
+  grid_wait(mode, voff);
   if (__ldg(mode) == kRecTileOrder)
     reduce_gather<D, NC>(voff, vrec, records, n_vert, dcoords, dcoef);
   else
@@ -523,22 +524,13 @@ cudaError_t launch_vertex_reduce(int dim, const BwdWorkspace& ws, int64_t n_vert
   if (n_vert == 0) return cudaSuccess;
   const int block = 256;
   const unsigned g = unsigned((n_vert + block - 1) / block);
-  if (dim == 2) {
-    if (ws.ncomp == 3)
-      vertex_reduce_kernel<2, 3><<<g, block, 0, stream>>>(ws.voff, ws.vrec, ws.mode, ws.records, n_vert, dcoords,
-                                                          dcoef);
-    else
-      vertex_reduce_kernel<2, 2><<<g, block, 0, stream>>>(ws.voff, ws.vrec, ws.mode, ws.records, n_vert, dcoords,
-                                                          nullptr);
-  } else {
-    if (ws.ncomp == 4)
-      vertex_reduce_kernel<3, 4><<<g, block, 0, stream>>>(ws.voff, ws.vrec, ws.mode, ws.records, n_vert, dcoords,
-                                                          dcoef);
-    else
-      vertex_reduce_kernel<3, 3><<<g, block, 0, stream>>>(ws.voff, ws.vrec, ws.mode, ws.records, n_vert, dcoords,
-                                                          nullptr);
-  }
-  return cudaGetLastError();
+  auto run = [&](auto kern) {
+    return launch_chained(kern, g, unsigned(block), 0, stream, static_cast<const int32_t*>(ws.voff),
+                          static_cast<const int32_t*>(ws.vrec), static_cast<const int32_t*>(ws.mode),
+                          static_cast<const float*>(ws.records), n_vert, dcoords, ws.ncomp > dim ? dcoef : nullptr);
+  };
+  if (dim == 2) return ws.ncomp == 3 ? run(vertex_reduce_kernel<2, 3>) : run(vertex_reduce_kernel<2, 2>);
+  return ws.ncomp == 4 ? run(vertex_reduce_kernel<3, 4>) : run(vertex_reduce_kernel<3, 3>);
 }
 
 }  // namespace fem

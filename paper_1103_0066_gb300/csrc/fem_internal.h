@@ -172,4 +172,45 @@ unsigned pipeline_grid(const void* kernel, int warps, size_t smem, int64_t n_ele
 // Raises the dynamic shared memory limit of a kernel when it needs more than 48 KB.
 cudaError_t ensure_smem(const void* kernel, size_t bytes);
 
+// Launch of a kernel that may be set up while the stream's previous kernel
+// ends (programmatic dependent launch): its CTAs take the places that the last
+// CTAs of that kernel leave, and grid_wait(), the kernel's first statement,
+// holds them until that kernel is complete and its writes are visible.  No
+// kernel here lets the next one begin earlier (launch_dependents): waiting
+// CTAs then took shared memory from running ones (128^3 cube, forward +
+// adjoint 478 -> 576 us, against 470 us without).
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                           const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+#ifdef __CUDACC__
+// Waits for the kernels before this one in the stream.  The index or pointers
+// that the kernel's first loads start from pass through the wait, so that the
+// compiler cannot move a read-only load above it (__ldg promises that nothing
+// writes the data, and a memory clobber does not order such loads).
+__device__ __forceinline__ void grid_wait(int64_t& index) {
+  asm volatile("griddepcontrol.wait;\n" : "+l"(index)::"memory");
+}
+template <class T, class U>
+__device__ __forceinline__ void grid_wait(const T*& p, const U*& q) {
+  asm volatile("griddepcontrol.wait;\n" : "+l"(p), "+l"(q)::"memory");
+}
+template <class T>
+__device__ __forceinline__ void grid_wait(int64_t& index, const T*& p) {
+  asm volatile("griddepcontrol.wait;\n" : "+l"(index), "+l"(p)::"memory");
+}
+#endif
+
 }  // namespace fem

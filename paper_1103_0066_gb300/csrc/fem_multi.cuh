@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, float, float>::threads,
   const int64_t T = P.tile_begin[P.n];
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t g = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(g);
   if (g >= T) return;  // warp-uniform
   int err = 0;
   int va[D + 1], vb[D + 1];
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(BwdShape<D, FORM, JAC>::threads, BwdShape<D, F
   const int64_t T = P.tile_begin[P.n];
   const int64_t S = int64_t(gridDim.x) * nwarps;
   int64_t g = int64_t(blockIdx.x) * nwarps + warp;
+  grid_wait(g);
   if (g >= T) return;  // warp-uniform: the kernel has no CTA-wide barrier
   int err = 0;
   int v1[D + 1], v2[D + 1], vc[D + 1];
@@ -243,7 +245,8 @@ __global__ void __launch_bounds__(BwdShape<D, FORM, JAC>::threads, BwdShape<D, F
 // single-mesh reduction.
 template <int D>
 __global__ void __launch_bounds__(kMultiRedBlock) vertex_reduce_multi_kernel(const __grid_constant__ RedMulti P) {
-  const int64_t b = blockIdx.x;
+  int64_t b = blockIdx.x;
+  grid_wait(b);
   int lo = 0, hi = P.n - 1;  // the last mesh whose first block is <= b
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -285,8 +288,7 @@ cudaError_t launch_fwd_multi_t(const FwdMulti& P, cudaStream_t st) {
   cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, T * 32, 0);
-  kern<<<grid, warps * 32, smem, st>>>(P);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, st, P);
 }
 
 template <int D, int FORM, int JAC>
@@ -300,16 +302,14 @@ cudaError_t launch_bwd_multi_t(const BwdMulti& P, cudaStream_t st) {
   cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, T * 32, 0);
-  kern<<<grid, warps * 32, smem, st>>>(P);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, unsigned(warps * 32), smem, st, P);
 }
 
 template <int D>
 cudaError_t launch_reduce_multi_t(const RedMulti& P, cudaStream_t st) {
   const int64_t blocks = P.blk_begin[P.n];
   if (blocks == 0) return cudaSuccess;
-  vertex_reduce_multi_kernel<D><<<unsigned(blocks), kMultiRedBlock, 0, st>>>(P);
-  return cudaGetLastError();
+  return launch_chained(vertex_reduce_multi_kernel<D>, unsigned(blocks), kMultiRedBlock, 0, st, P);
 }
 
 }  // namespace fem
