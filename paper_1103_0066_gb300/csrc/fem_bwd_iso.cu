@@ -27,7 +27,8 @@
 // the arithmetic; the next connectivity is loaded with it.
 // P2 tets, 64^3 cube: 343 us with the contraction over 78 folded slot pairs,
 // 291 us by the structure of K, 240 us with the copy ahead and 12 warps per SM
-// (8 at the 250 registers it takes unbounded: 244 us; 16 spill: 310 us).
+// (8 at the 250 registers it takes unbounded: 244 us; 16 spill: 310 us), 221
+// us with dA copied unpadded.
 // Bound by instruction issue and the latency of the geometry's loads (issue
 // 56% active at 11.4 warps).  P1 tets: 102 us.
 #include "fem_iso_adj.cuh"

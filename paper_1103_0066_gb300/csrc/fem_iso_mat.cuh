@@ -60,43 +60,37 @@ __host__ __device__ __forceinline__ float iso_dot(const float* u, const float* v
 }
 
 // P1: acc[(i, j)] = (D+4)(D+3) b of the pair (i, j), b = P_i . P_j + sum_k p_{k,i} . p_{k,j}
-// with P_i = sum_k p_{k,i}; the entries of index 0 from the zero row sums.
+// with P_i = sum_k p_{k,i}.  Every pair directly, the small terms first: taking
+// the entries of index 0 from the zero row sums doubles the largest error
+// (8.0e-7 against 4.5e-7 of an element's largest entry, warped 128^3 cube).
 template <int D>
 __host__ __device__ __forceinline__ void iso_matrix_p1(const float (&ji)[D + 1][D][D], float* acc) {
   constexpr int NV = D + 1;
-  float P[D][D];
+  float p0[NV][D], P[NV][D];
+  iso_p0<D>(ji, p0);
 #pragma unroll
-  for (int a = 0; a < D; ++a)
+  for (int a = 0; a < NV; ++a)
 #pragma unroll
     for (int al = 0; al < D; ++al) {
-      float s = ji[0][a][al];
+      float s = a ? ji[0][a ? a - 1 : 0][al] : p0[0][al];
 #pragma unroll
-      for (int k = 1; k < NV; ++k) s += ji[k][a][al];
+      for (int k = 1; k < NV; ++k) s += a ? ji[k][a ? a - 1 : 0][al] : p0[k][al];
       P[a][al] = s;
     }
-  float row[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) row[i] = 0.f;
-#pragma unroll
-  for (int x = 1; x < NV; ++x)
+  for (int x = 0; x < NV; ++x)
 #pragma unroll
     for (int y = x; y < NV; ++y) {
-      float b = iso_dot<D>(P[x - 1], P[y - 1]);
+      float b = 0.f;  // the small terms first, the large one last
 #pragma unroll
-      for (int k = 0; k < NV; ++k)
+      for (int k = 0; k < NV; ++k) {
+        const float* kx = x ? ji[k][x ? x - 1 : 0] : p0[k];
+        const float* ky = y ? ji[k][y ? y - 1 : 0] : p0[k];
 #pragma unroll
-        for (int al = 0; al < D; ++al) b = fmaf(ji[k][x - 1][al], ji[k][y - 1][al], b);
-      b *= IsoMat<D>::n2;
-      acc[pair_index(x, y, NV)] = b;
-      row[x] += b;
-      if (x != y) row[y] += b;
+        for (int al = 0; al < D; ++al) b = fmaf(kx[al], ky[al], b);
+      }
+      acc[pair_index(x, y, NV)] = IsoMat<D>::n2 * (b + iso_dot<D>(P[x], P[y]));
     }
-#pragma unroll
-  for (int x = 1; x < NV; ++x) {
-    acc[pair_index(0, x, NV)] = -row[x];
-    row[0] += row[x];
-  }
-  acc[0] = row[0];
 }
 
 // P2: acc[(i, j)] of the upper triangle, without the common factor.
