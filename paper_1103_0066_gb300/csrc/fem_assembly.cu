@@ -44,8 +44,7 @@ constexpr int kMaxCols = 255;   // distinct columns per row (one-byte positions)
 constexpr int kFastCols = 32;   // columns of a row accumulated in shared memory
 constexpr int kPatWarps = 4;
 
-// Lanes a row takes (one per component of its blocks) and rows of a row block.
-__host__ __device__ constexpr int row_lanes(int B) { return B * B; }
+// Rows of a row block: a row takes a lane per component of its blocks.
 __host__ __device__ constexpr int block_rows(int B) { return 32 / (B * B); }
 // Marks in a byte of a slot's column word (scalar forms): the contribution is
 // the first / the last one of its 32-element tile to its entry.
