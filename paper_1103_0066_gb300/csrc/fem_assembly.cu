@@ -42,6 +42,7 @@ namespace {
 constexpr int kRowCap = 512;    // candidate columns per row (incidences x (d+1))
 constexpr int kMaxCols = 255;   // distinct columns per row (one-byte positions)
 constexpr int kFastCols = 32;   // columns of a row accumulated in shared memory
+constexpr int kPadCol = kFastCols;  // the column of padded slots
 constexpr int kPatWarps = 4;
 
 // Rows of a row block: a row takes a lane per component of its blocks.
@@ -159,9 +160,10 @@ __global__ void __launch_bounds__(kPatWarps * 32)
 
 // ------------------------------------------------------------------ row blocks (P1 forms and elasticity)
 
-// Steps of each row block: its longest row's incidences; 0 where the kernel
-// has to scan instead, because a row has more than kFastCols columns or an
-// element of it lists the row's vertices twice (its positions then coincide).
+// Steps of each row block: the incidences of its longest row.  A row of more
+// than kFastCols columns is scanned: among the 32 rows of a scalar block alone
+// (it gets padding here), a block of three or eight rows as a whole (steps 0),
+// like one where an element lists a vertex twice (its positions then coincide).
 template <int NV, int B>
 __global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ row_ptr,
                                    const uint8_t* __restrict__ colpos, int64_t n_vert, int32_t* steps) {
@@ -171,7 +173,10 @@ __global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const in
     int n = 0;
     bool fast = true;
     for (int64_t v = b * G; v < (b + 1) * G && v < n_vert; ++v) {
-      fast &= row_ptr[v + 1] - row_ptr[v] <= kFastCols;
+      if (row_ptr[v + 1] - row_ptr[v] > kFastCols) {
+        fast &= B == 1;
+        continue;
+      }
       const int c = inc_off[v + 1] - inc_off[v];
       n = c > n ? c : n;
       if constexpr (B > 1)  // the scalar forms refuse such elements
@@ -192,7 +197,8 @@ __global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const in
 // at them.  first marks are counted: one per (tile, entry), the tile records.
 template <int NV, int B>
 __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
-                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ blk_off,
+                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
+                                  const int32_t* __restrict__ blk_off,
                                   int64_t n_vert, int64_t slot_cap, int2* __restrict__ slots, int32_t* n_records) {
   constexpr int G = block_rows(B);
   const int64_t nblk = (n_vert + G - 1) / G;
@@ -202,8 +208,9 @@ __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int
     const int64_t b = v / G;
     const int32_t s0 = blk_off[b], steps = blk_off[b + 1] - s0;
     const int32_t t0 = inc_off[v], n = inc_off[v + 1] - t0;
+    const bool fits = row_ptr[v + 1] - row_ptr[v] <= kFastCols;
     for (int k = 0; k < (steps > n ? steps : n); ++k) {
-      int2 q = make_int2(-1, 0);
+      int2 q = make_int2(-1, kPadCol * 0x01010101);
       if (k < n) {
         const int32_t t = t0 + k;
         q.x = inc[t];
@@ -228,7 +235,8 @@ __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int
         }
         q.y = int(w);
       }
-      if (room && k < steps) slots[(int64_t(s0) + k) * G + (v - b * G)] = q;
+      if (room && k < steps)
+        slots[(int64_t(s0) + k) * G + (v - b * G)] = fits ? q : make_int2(-1, kPadCol * 0x01010101);
     }
   }
   if constexpr (B == 1) {
@@ -256,7 +264,6 @@ __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int
 // 8 steps in flight and four CTAs per SM the rest of L1 keeps the sectors that
 // a later row needs (four steps and eight CTAs: 162 us; on triangles the
 // shorter rows prefer the latter, 42 against 46 us at 600 x 600).
-constexpr int kPadCol = kFastCols;
 template <int B>
 struct BlockPlan {
   static constexpr bool staged = B == 1;
@@ -320,6 +327,29 @@ __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ct
   const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
   // the sums are zero at the start of every block: zeroed here, and again as they are read out
   for (int c = 0; c <= kFastCols; ++c) *reinterpret_cast<float*>(mine + c * 128) = 0.f;
+  // a lane per value, every incidence of the row looked at
+  auto scan_row = [&](int64_t r) {
+    const int32_t rp = __ldg(row_ptr + r), t0 = __ldg(inc_off + r), t1 = __ldg(inc_off + r + 1);
+    const int words = (__ldg(row_ptr + r + 1) - rp) * BB;
+    for (int x = lane; x < words; x += 32) {
+      const int c = x / BB, c1 = (x % BB) / B, c2 = x % B;
+      float sum = 0.f, part = 0.f;
+      int tile = -1;
+      for (int32_t t = t0; t < t1; ++t) {
+        const int32_t s = __ldg(inc + t);
+        const float* src = A + int64_t(s / NV) * (N * N) + (c1 * NV + s % NV) * N + c2 * NV;
+        if (B == 1 && (s / NV) >> 5 != tile) {
+          sum += part;
+          part = 0.f;
+          tile = (s / NV) >> 5;
+        }
+#pragma unroll
+        for (int j = 0; j < NV; ++j)
+          if (__ldg(colpos + int64_t(t) * NV + j) == c) (B == 1 ? part : sum) += __ldg(src + j);
+      }
+      val[int64_t(rp) * BB + x] = sum + part;
+    }
+  };
   for (; b < nblk; b += int64_t(gridDim.x) * BP::warps) {
     const int64_t r0 = b * G;
     const int nr = int(n_vert - r0 < G ? n_vert - r0 : G);
@@ -329,7 +359,10 @@ __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ct
     if (room && steps > 0) {
       const bool live = g < nr;
       const int32_t rb = live ? __ldg(row_ptr + r0 + g) : 0;
-      const int len = live ? __ldg(row_ptr + r0 + g + 1) - rb : 0;
+      const int row_len = live ? __ldg(row_ptr + r0 + g + 1) - rb : 0;
+      // scalar forms: a long row's slots are padding, it is scanned below
+      const uint32_t long_lanes = B == 1 ? __ballot_sync(0xffffffffu, row_len > kFastCols) : 0u;
+      const int len = B == 1 && row_len > kFastCols ? 0 : row_len;
       const int2* sl = slots + int64_t(s0) * G + g;
       int2 ahead[U];  // slots of the next batch to load
       auto load_slots = [&](int k0) {
@@ -420,7 +453,7 @@ __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ct
         }
       }
       const int maxlen = __reduce_max_sync(0xffffffffu, len);
-      if constexpr (B == 1) {
+      if (B == 1 && long_lanes == 0) {
         // pack the rows' values where the open tile sums were (all closed) and store them coalesced
         __syncwarp();
         float* pack = reinterpret_cast<float*>(wbase + kPart);
@@ -443,30 +476,10 @@ __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ct
           }
       }
       __syncwarp();  // the sums are the next block's
+      if constexpr (B == 1)
+        for (uint32_t left = long_lanes; left; left &= left - 1) scan_row(r0 + __ffs(left) - 1);
     } else {
-      // scanning path: a lane per value, every incidence of the row looked at
-      for (int h = 0; h < nr; ++h) {
-        const int32_t rp = __ldg(row_ptr + r0 + h), t0 = __ldg(inc_off + r0 + h), t1 = __ldg(inc_off + r0 + h + 1);
-        const int words = (__ldg(row_ptr + r0 + h + 1) - rp) * BB;
-        for (int x = lane; x < words; x += 32) {
-          const int c = x / BB, c1 = (x % BB) / B, c2 = x % B;
-          float sum = 0.f, part = 0.f;
-          int tile = -1;
-          for (int32_t t = t0; t < t1; ++t) {
-            const int32_t s = __ldg(inc + t);
-            const float* src = A + int64_t(s / NV) * (N * N) + (c1 * NV + s % NV) * N + c2 * NV;
-            if (B == 1 && (s / NV) >> 5 != tile) {
-              sum += part;
-              part = 0.f;
-              tile = (s / NV) >> 5;
-            }
-#pragma unroll
-            for (int j = 0; j < NV; ++j)
-              if (__ldg(colpos + int64_t(t) * NV + j) == c) (B == 1 ? part : sum) += __ldg(src + j);
-          }
-          val[int64_t(rp) * BB + x] = sum + part;
-        }
-      }
+      for (int h = 0; h < nr; ++h) scan_row(r0 + h);
     }
   }
 }
@@ -551,8 +564,8 @@ cudaError_t launch_row_blocks(int64_t n_vert, const AsmLayout& L, cudaStream_t s
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = launch_exclusive_scan(L.cursor, nblk, L.partials, L.blk_off, st);
   if (e != cudaSuccess) return e;
-  block_fill_kernel<NV, B><<<grid_of(n_vert, 256), 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.blk_off, n_vert,
-                                                                 L.slot_cap, L.slots, L.flag + 1);
+  block_fill_kernel<NV, B><<<grid_of(n_vert, 256), 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off,
+                                                                 n_vert, L.slot_cap, L.slots, L.flag + 1);
   return cudaGetLastError();
 }
 
