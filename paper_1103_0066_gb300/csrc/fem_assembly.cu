@@ -13,12 +13,14 @@
 //                distinct ones (the row's columns, increasing), and stores for
 //                every incidence t and local vertex j the position of
 //                conn[e][j] among them (colpos, one byte)
-//   row blocks : (P1 forms and elasticity) the incidences of 32 / B^2
-//                consecutive rows, padded to the longest row of the block and
-//                interleaved, so that the lanes of a warp read them coalesced
+//   row blocks : (P1 forms and elasticity) rows that share elements, of like
+//                length, in blocks of 32 / B^2 (16 for rows of 33 to 63
+//                columns of the scalar forms); their incidences, padded to the
+//                longest row of the block and interleaved, so that the lanes
+//                of a warp read them coalesced.  Longer rows are listed.
 // Assembly (fem_assemble), P1 forms and elasticity: one kernel, a warp per row
-// block, a lane per row and block component.  A lane walks its row's
-// incidences in element order, reads the element row's NV entries of its
+// block, a lane per row and block component (a few lanes per long row).  A lane
+// walks its row's incidences in element order, reads the element row's NV entries of its
 // component (16 bytes on tets) and adds them to its own column sums in shared
 // memory.  No two lanes share a sum, so the order of every sum is the lane's
 // program order:
@@ -41,12 +43,33 @@ namespace {
 
 constexpr int kRowCap = 512;    // candidate columns per row (incidences x (d+1))
 constexpr int kMaxCols = 255;   // distinct columns per row (one-byte positions)
-constexpr int kFastCols = 32;   // columns of a row accumulated in shared memory
-constexpr int kPadCol = kFastCols;  // the column of padded slots
 constexpr int kPatWarps = 4;
 
-// Rows of a row block: a row takes a lane per component of its blocks.
-__host__ __device__ constexpr int block_rows(int B) { return 32 / (B * B); }
+// Kinds of rows by the room that their sums take in a warp's shared memory:
+// short ones, up to 32 columns, have a block of 32 / B^2 rows, a lane per
+// component of a row's blocks; the wide rows of the scalar forms, 33 to 63
+// columns, a block of 16; longer rows have no blocks (LongPlan).  Rows of more
+// than 32 incidences go with the wide ones, which start first: among short rows
+// they come late and hold a warp when the others are done (barycentric 40^3
+// cube, vertices numbered at random, 95 -> 87 us).
+enum : int { ROW_SHORT = 0, ROW_WIDE = 1, ROW_LONG = 2 };
+constexpr int kWideRows = 16;
+template <int B, int KIND>
+struct BlockRows {
+  static constexpr int rows = KIND == ROW_WIDE ? kWideRows : 32 / (B * B);
+  static constexpr int cols = KIND == ROW_WIDE ? 63 : 32;  // and a column for padded slots, which add zeros to it
+  static constexpr int shift = KIND == ROW_WIDE ? 6 : 7;   // log2 of the bytes between a lane's columns
+  // a step's slots in units of blk_off
+  static constexpr int unit = B == 1 ? 16 : rows, units = rows / unit;
+  // Blocks and rows of a window, within which the build may order the rows by
+  // their length: a prime number of blocks, so that the first blocks of the
+  // windows, the longest ones, fall on different warps of the grid (with 32
+  // blocks a window and 2432 warps the same 76 took them all: barycentric 40^3
+  // cube, vertices numbered at random, 152 us against 122).
+  static constexpr int win_blocks = B == 1 ? 31 : B == 2 ? 127 : 251, win_rows = win_blocks * rows;
+};
+constexpr uint32_t pad_word(int cols) { return uint32_t(cols) * 0x01010101u; }
+
 // Marks in a byte of a slot's column word (scalar forms): the contribution is
 // the first / the last one of its 32-element tile to its entry.
 constexpr uint32_t kFirst = 0x40, kLast = 0x80;
@@ -160,33 +183,165 @@ __global__ void __launch_bounds__(kPatWarps * 32)
 
 // ------------------------------------------------------------------ row blocks (P1 forms and elasticity)
 
-// Steps of each row block: the incidences of its longest row.  A row of more
-// than kFastCols columns is scanned: among the 32 rows of a scalar block alone
-// (it gets padding here), a block of three or eight rows as a whole (steps 0),
-// like one where an element lists a vertex twice (its positions then coincide).
+// Most incidences of a row (row_pattern_kernel refuses more).
+__host__ __device__ constexpr int max_incidences(int nv) { return kRowCap / nv; }
+
+// An element of row v lists a vertex twice (its column positions coincide).
+template <int NV>
+__device__ __forceinline__ bool row_repeats(const int32_t* inc_off, const uint8_t* colpos, int64_t v) {
+  for (int32_t t = inc_off[v]; t < inc_off[v + 1]; ++t)
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+#pragma unroll
+      for (int j = i + 1; j < NV; ++j)
+        if (colpos[int64_t(t) * NV + i] == colpos[int64_t(t) * NV + j]) return true;
+  return false;
+}
+
+// The order of the rows.  The rows of a warp should share elements, whose
+// matrices they then read from the same lines; so the rows go by their number
+// where rows numbered one after the other mostly are neighbours in the element
+// list too, else by their first incidence.  (80^3 cube, vertices numbered at
+// random: scalar 145 us by number, 100 by incidence, 87 numbered in order;
+// elasticity 930, 444 and 437.)  Rows without elements drop out.  Long rows
+// have no blocks, and neither have rows where an element repeats a vertex (the
+// scalar forms refuse such elements).
+
+// near[0], near[1]: the vertices v with elements that v + 1 has too, and those
+// among them whose first incidences lie within kNear of each other.
+constexpr int kNear = 512;
+
+__global__ void row_near_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc, int64_t n_vert,
+                                int32_t* near) {
+  int pairs = 0, close = 0;
+  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v + 1 < n_vert;
+       v += int64_t(gridDim.x) * blockDim.x) {
+    const int32_t a = inc_off[v], b = inc_off[v + 1];
+    if (a == b || b == inc_off[v + 2]) continue;
+    ++pairs;
+    close += abs(inc[a] - inc[b]) <= kNear;
+  }
+  __syncwarp();
+  pairs = __reduce_add_sync(0xffffffffu, pairs);
+  close = __reduce_add_sync(0xffffffffu, close);
+  if (pairs && (threadIdx.x & 31) == 0) {
+    atomicAdd(near, pairs);
+    atomicAdd(near + 1, close);
+  }
+}
+
+// The place of row v among the rows: its number or its first incidence.
+__device__ __forceinline__ int32_t row_key(const int32_t* inc_off, const int32_t* inc, int by_number, int64_t v) {
+  return by_number ? int32_t(v) : inc[inc_off[v]];
+}
+
 template <int NV, int B>
-__global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ row_ptr,
-                                   const uint8_t* __restrict__ colpos, int64_t n_vert, int32_t* steps) {
-  constexpr int G = block_rows(B);
-  const int64_t nblk = (n_vert + G - 1) / G;
-  for (int64_t b = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; b < nblk; b += int64_t(gridDim.x) * blockDim.x) {
-    int n = 0;
-    bool fast = true;
-    for (int64_t v = b * G; v < (b + 1) * G && v < n_vert; ++v) {
-      if (row_ptr[v + 1] - row_ptr[v] > kFastCols) {
-        fast &= B == 1;
-        continue;
-      }
-      const int c = inc_off[v + 1] - inc_off[v];
-      n = c > n ? c : n;
-      if constexpr (B > 1)  // the scalar forms refuse such elements
-        for (int32_t t = inc_off[v]; fast && t < inc_off[v + 1]; ++t)
-#pragma unroll
-          for (int i = 0; i < NV; ++i)
-#pragma unroll
-            for (int j = i + 1; j < NV; ++j) fast &= colpos[int64_t(t) * NV + i] != colpos[int64_t(t) * NV + j];
+__device__ __forceinline__ int row_kind(const int32_t* inc_off, const uint8_t* colpos, const int32_t* row_ptr,
+                                        int repeats, int64_t v) {
+  const int len = row_ptr[v + 1] - row_ptr[v];
+  const bool room = len <= BlockRows<B, ROW_SHORT>::cols;
+  if (B > 1) return room && !(repeats && row_repeats<NV>(inc_off, colpos, v)) ? ROW_SHORT : ROW_LONG;
+  if (len > BlockRows<B, ROW_WIDE>::cols) return ROW_LONG;
+  return room && inc_off[v + 1] - inc_off[v] <= 32 ? ROW_SHORT : ROW_WIDE;
+}
+
+// flag[key] = 1 for every row of the kind.
+template <int NV, int B, int KIND>
+__global__ void row_flag_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                                const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
+                                int by_number, int repeats, int64_t n_vert, int32_t* __restrict__ flag) {
+  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n_vert; v += int64_t(gridDim.x) * blockDim.x)
+    if (inc_off[v + 1] > inc_off[v] && row_kind<NV, B>(inc_off, colpos, row_ptr, repeats, v) == KIND)
+      flag[row_key(inc_off, inc, by_number, v)] = 1;
+}
+
+// The flagged rows at the exclusive scan foff of their flags (long rows as ~v
+// where an element repeats a vertex).
+template <int NV, int B, int KIND>
+__global__ void row_place_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                                 const uint8_t* __restrict__ colpos, const int32_t* __restrict__ foff,
+                                 int by_number, int repeats, int64_t n_vert, int32_t* __restrict__ rows) {
+  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n_vert; v += int64_t(gridDim.x) * blockDim.x) {
+    if (inc_off[v + 1] == inc_off[v]) continue;
+    const int32_t s = row_key(inc_off, inc, by_number, v);
+    if (foff[s + 1] > foff[s])
+      rows[foff[s]] = int32_t(KIND == ROW_LONG && repeats && row_repeats<NV>(inc_off, colpos, v) ? ~v : v);
+  }
+}
+
+// Rows of each kind, and where the blocks of the kinds begin: the wide ones first.
+struct RowCounts {
+  int32_t n_long, n_wide, n_short;
+  __device__ int wide_blocks() const { return int((int64_t(n_wide) + kWideRows - 1) / kWideRows); }
+  template <int B>
+  __device__ int blocks() const {
+    constexpr int G = BlockRows<B, ROW_SHORT>::rows;
+    return wide_blocks() + int((int64_t(n_short) + G - 1) / G);
+  }
+};
+
+// The blocks of a kind of rows, a CTA per window: the rows in their order where
+// that pads the window's slots by no more than half, else by their incidence
+// counts, the largest first (equal ones in their order).  order: the row, or -1
+// behind the last one; steps: the incidences of each block's longest row, in
+// units of slots.
+//
+// Sorted, a block's slots number at most the incidences of the block before
+// it, so a window is padded by at most its rows' share of the largest count.
+template <int NV, int B, int KIND>
+__global__ void __launch_bounds__(256)
+    block_order_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ rows,
+                       const RowCounts* __restrict__ counts, int32_t* __restrict__ order, int32_t* __restrict__ steps) {
+  using K = BlockRows<B, KIND>;
+  constexpr int G = K::rows, W = K::win_rows, P = 1024;
+  static_assert(W <= P && W % G == 0 && max_incidences(NV) < 256, "keys: 255 - count, then the row");
+  __shared__ uint32_t key[P];
+  __shared__ int padded, total;
+  const int tid = threadIdx.x;
+  const int64_t n = KIND == ROW_WIDE ? counts->n_wide : counts->n_short;
+  if (KIND == ROW_SHORT) {
+    steps += counts->wide_blocks();
+    order += int64_t(counts->wide_blocks()) * kWideRows;
+  }
+  for (int64_t r0 = int64_t(blockIdx.x) * W; r0 < n; r0 += int64_t(gridDim.x) * W) {
+    if (tid == 0) padded = total = 0;
+    for (int i = tid; i < P; i += 256) {
+      const int64_t v = i < W && r0 + i < n ? rows[r0 + i] : -1;
+      key[i] = (uint32_t(255 - (v < 0 ? 0 : inc_off[v + 1] - inc_off[v])) << 16) | uint32_t(i);
     }
-    steps[b] = fast ? n : 0;
+    __syncthreads();
+    for (int k = tid; k < W / G; k += 256) {
+      int top = 0, sum = 0;
+      for (int i = k * G; i < (k + 1) * G; ++i) {
+        const int c = 255 - int(key[i] >> 16);
+        top = c > top ? c : top;
+        sum += c;
+      }
+      atomicAdd(&padded, G * top);
+      atomicAdd(&total, sum);
+    }
+    __syncthreads();
+    if (2 * padded > 3 * total)
+      for (int k2 = 2; k2 <= P; k2 <<= 1)
+        for (int jj = k2 >> 1; jj > 0; jj >>= 1) {
+          for (int i = tid; i < P; i += 256) {
+            const int ixj = i ^ jj;
+            const uint32_t x = key[i], y = ixj > i ? key[ixj] : 0;
+            if (ixj > i && (x > y) == ((i & k2) == 0)) {
+              key[i] = y;
+              key[ixj] = x;
+            }
+          }
+          __syncthreads();
+        }
+    const int nb = int(((n - r0 < W ? n - r0 : W) + G - 1) / G);
+    for (int i = tid; i < nb * G; i += 256) order[r0 + i] = r0 + i < n ? rows[r0 + int(key[i] & 0xFFFFu)] : -1;
+    for (int k = tid; k < nb; k += 256) {
+      int top = 0;
+      for (int i = k * G; i < (k + 1) * G; ++i) top = max(top, 255 - int(key[i] >> 16));
+      steps[r0 / G + k] = top * K::units;
+    }
+    __syncthreads();  // the keys are the next window's
   }
 }
 
@@ -194,52 +349,59 @@ __global__ void block_steps_kernel(const int32_t* __restrict__ inc_off, const in
 // j: the column position, for the scalar forms with the tile marks), padded
 // with element slot -1 to the block's steps.  A tile's incidences of one row
 // are neighbours (the list is in element order), so the marks come from a look
-// at them.  first marks are counted: one per (tile, entry), the tile records.
-template <int NV, int B>
+// at them.  first marks are counted, of the long rows too: one per (tile,
+// entry), the tile records.
+template <int NV, int B, int KIND>
 __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
-                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                                  const int32_t* __restrict__ blk_off,
-                                  int64_t n_vert, int64_t slot_cap, int2* __restrict__ slots, int32_t* n_records) {
-  constexpr int G = block_rows(B);
-  const int64_t nblk = (n_vert + G - 1) / G;
-  const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
+                                  const uint8_t* __restrict__ colpos, const int32_t* __restrict__ order,
+                                  const int32_t* __restrict__ blk_off, const int32_t* __restrict__ long_rows,
+                                  const RowCounts* __restrict__ counts, int2* __restrict__ slots, int32_t* n_records) {
+  using K = BlockRows<B, KIND>;
+  constexpr int G = K::rows;
+  const int b0 = KIND == ROW_WIDE ? 0 : counts->wide_blocks();
+  const int64_t at_end = int64_t(KIND == ROW_WIDE ? counts->wide_blocks() : counts->template blocks<B>() - b0) * G;
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  blk_off += b0;
+  order += int64_t(b0) * kWideRows;
   int nrec = 0;
-  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n_vert; v += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t b = v / G;
-    const int32_t s0 = blk_off[b], steps = blk_off[b + 1] - s0;
-    const int32_t t0 = inc_off[v], n = inc_off[v + 1] - t0;
-    const bool fits = row_ptr[v + 1] - row_ptr[v] <= kFastCols;
-    for (int k = 0; k < (steps > n ? steps : n); ++k) {
-      int2 q = make_int2(-1, kPadCol * 0x01010101);
-      if (k < n) {
-        const int32_t t = t0 + k;
-        q.x = inc[t];
-        uint32_t w = 0;
-        const int32_t tile = (q.x / NV) >> 5;
+  // the word of incidence t of the row with incidences [t0, t1)
+  auto word = [&](int32_t t, int32_t t0, int32_t t1) {
+    uint32_t w = 0;
+    const int32_t tile = (inc[t] / NV) >> 5;
 #pragma unroll
-        for (int j = 0; j < NV; ++j) {
-          const uint32_t c = colpos[int64_t(t) * NV + j];
-          uint32_t m = c & 0x3Fu;  // rows of more columns take the scanning path
-          if constexpr (B == 1) {
-            bool first = true, last = true;
-            for (int32_t u = t - 1; first && u >= t0 && (inc[u] / NV) >> 5 == tile; --u)
+    for (int j = 0; j < NV; ++j) {
+      const uint32_t c = colpos[int64_t(t) * NV + j];
+      uint32_t m = c & 0x3Fu;  // long rows take no words
+      if constexpr (B == 1) {
+        bool first = true, last = true;
+        for (int32_t u = t - 1; first && u >= t0 && (inc[u] / NV) >> 5 == tile; --u)
 #pragma unroll
-              for (int i = 0; i < NV; ++i) first &= colpos[int64_t(u) * NV + i] != c;
-            for (int32_t u = t + 1; last && u < t0 + n && (inc[u] / NV) >> 5 == tile; ++u)
+          for (int i = 0; i < NV; ++i) first &= colpos[int64_t(u) * NV + i] != c;
+        for (int32_t u = t + 1; last && u < t1 && (inc[u] / NV) >> 5 == tile; ++u)
 #pragma unroll
-              for (int i = 0; i < NV; ++i) last &= colpos[int64_t(u) * NV + i] != c;
-            m |= (first ? kFirst : 0u) | (last ? kLast : 0u);
-            nrec += first;
-          }
-          w |= m << (8 * j);
-        }
-        q.y = int(w);
+          for (int i = 0; i < NV; ++i) last &= colpos[int64_t(u) * NV + i] != c;
+        m |= (first ? kFirst : 0u) | (last ? kLast : 0u);
+        nrec += first;
       }
-      if (room && k < steps)
-        slots[(int64_t(s0) + k) * G + (v - b * G)] = fits ? q : make_int2(-1, kPadCol * 0x01010101);
+      w |= m << (8 * j);
     }
+    return w;
+  };
+  for (int64_t at = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; at < at_end; at += stride) {
+    const int64_t b = at / G, v = order[at];
+    const int64_t s0 = int64_t(blk_off[b]) * K::unit;
+    const int steps = (blk_off[b + 1] - blk_off[b]) / K::units;
+    const int32_t t0 = v < 0 ? 0 : inc_off[v], t1 = v < 0 ? 0 : inc_off[v + 1];
+    for (int k = 0; k < steps; ++k)
+      slots[s0 + int64_t(k) * G + (at - b * G)] =
+          k < t1 - t0 ? make_int2(inc[t0 + k], int(word(t0 + k, t0, t1))) : make_int2(-1, int(pad_word(K::cols)));
   }
   if constexpr (B == 1) {
+    const int64_t n_long = KIND == ROW_SHORT ? counts->n_long : 0;
+    for (int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; q < n_long; q += stride) {
+      const int64_t v = long_rows[q];
+      for (int32_t t = inc_off[v]; t < inc_off[v + 1]; ++t) word(t, inc_off[v], inc_off[v + 1]);
+    }
     __syncwarp();
     nrec = __reduce_add_sync(0xffffffffu, nrec);
     if (nrec && (threadIdx.x & 31) == 0) atomicAdd(n_records, nrec);
@@ -248,8 +410,9 @@ __global__ void block_fill_kernel(const int32_t* __restrict__ inc_off, const int
 
 // Shared memory of a warp: [sums][open tile sums, scalar forms][stage].  The
 // sum of column c of lane l lies at c * 32 + l, a lane's sums in its own bank.
-// Padded slots add zeros to a column of their own (kPadCol), which keeps the
-// loop free of branches.
+// Padded slots add zeros to a column of their own, which keeps the loop free of
+// branches.  (In a block of wide rows column c of lane l lies at c * 16 + l, and
+// the upper lanes have padded slots only.)
 //
 // Scalar forms: the element rows come through a stage of two batches of two
 // steps with 16-byte cp.async, which goes around L1.  A scattered load takes a
@@ -271,7 +434,7 @@ struct BlockPlan {
   static constexpr int min_ctas = staged ? 1 : B == 3 ? 4 : 8;
   static constexpr int batch = staged ? 2 : B == 3 ? 8 : 4;  // steps loaded together
   static constexpr int stages = staged ? 2 : 1;
-  static constexpr size_t sums = size_t(kFastCols + 1) * 128;
+  static constexpr size_t sums = size_t(BlockRows<B, ROW_SHORT>::cols + 1) * 128;
   static constexpr size_t stage_off = (B == 1 ? 2 : 1) * sums;
   static constexpr size_t per_warp = stage_off + (staged ? size_t(stages) * batch * 512 : 0);
   static constexpr size_t smem = warps * per_warp;
@@ -293,6 +456,326 @@ __device__ __forceinline__ void copy_piece(void* dst, const float* A, int64_t of
   }
 }
 
+// Long rows (more than 63 columns, 32 of blocks): 32 / (NV B) of them per warp, a lane per column block component
+// (c2, j), NV B neighbouring floats of an element row.  A lane walks the row's
+// incidences in element order and adds its B values to the sums of its column
+// in shared memory; the columns of an element differ, so a step has no
+// conflicts.  The scalar forms keep, per column, the sum of the closed tiles,
+// that of the open tile, and the open tile's number.  Rows of more columns
+// than a warp has room for are walked once per range of columns; a row where
+// an element repeats a vertex (~v in the list) is taken value by value.
+template <int NV, int B>
+struct LongPlan {
+  static constexpr int lanes = NV * B, rows = 32 / lanes;
+  static constexpr int words = int(BlockPlan<B>::per_warp / 4 / rows);  // of shared memory, per row
+  static constexpr int per_col = B == 1 ? 3 : B * B;
+  static constexpr int batch = B == 1 ? 8 : 4;  // incidences loaded together
+  static constexpr int cols = (words / per_col - 1) | 1;  // an odd number of columns spreads the rows over the banks
+  static_assert(B > 1 || cols < 128, "seven bits of a word");
+};
+
+template <int NV, int B>
+__device__ __forceinline__ void assemble_long_rows(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
+                                                   const uint8_t* __restrict__ colpos,
+                                                   const int32_t* __restrict__ row_ptr,
+                                                   const int32_t* __restrict__ long_rows, int n_long, int64_t unit,
+                                                   const float* __restrict__ A, float* __restrict__ val, float* sm,
+                                                   int lane) {
+  using LP = LongPlan<NV, B>;
+  constexpr int BB = B * B, N = NV * B, L = LP::lanes, R = LP::rows, C = LP::cols, U = LP::batch;
+  const int g = lane / L, l = lane % L, j = l % NV;
+  const int64_t q = unit * R + g;
+  const int32_t v = g < R && q < n_long ? __ldg(long_rows + q) : -1;
+  const int32_t rb = v < 0 ? 0 : __ldg(row_ptr + v), len = v < 0 ? 0 : __ldg(row_ptr + v + 1) - rb;
+  const int32_t t0 = v < 0 ? 0 : __ldg(inc_off + v), n = v < 0 ? 0 : __ldg(inc_off + v + 1) - t0;
+  const int steps = __reduce_max_sync(0xffffffffu, n), maxlen = __reduce_max_sync(0xffffffffu, len);
+  float* sum = sm + (g < R ? g : 0) * LP::words;  // [column][BB]; scalar forms: closed tiles, open tile, its number
+  int* tile = reinterpret_cast<int*>(sum + 2 * C);
+  for (int c0 = 0; c0 < maxlen; c0 += C) {
+    const int here = len <= c0 ? 0 : len - c0 < C ? len - c0 : C;  // columns of this range
+    for (int x = l; x < here * (B == 1 ? 1 : BB); x += L) {
+      sum[x] = 0.f;
+      if (B == 1) sum[C + x] = 0.f, tile[x] = -1;
+    }
+    __syncwarp();
+    int32_t sl[U];  // slots and columns of the next batch
+    int col[U];
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool on = k0 + u < n;
+        sl[u] = on ? __ldg(inc + t0 + k0 + u) : 0;
+        col[u] = on ? int(__ldg(colpos + (int64_t(t0) + k0 + u) * NV + j)) - c0 : -1;
+      }
+    };
+    load(0);
+    for (int k0 = 0; k0 < steps; k0 += U) {
+      int32_t at[U];
+      float a[U][B];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool in = col[u] >= 0 && col[u] < here;
+        at[u] = in ? (B == 1 ? (((sl[u] / NV) >> 5) << 7) | col[u] : col[u]) : -1;  // the tile, the column
+        const float* src = A + int64_t(sl[u] / NV) * (N * N) + (sl[u] % NV) * N + l;
+#pragma unroll
+        for (int c = 0; c < B; ++c) a[u][c] = in ? __ldg(src + c * NV * N) : 0.f;
+      }
+      load(k0 + U);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (at[u] >= 0) {
+          if constexpr (B == 1) {
+            const int c = at[u] & 127;
+            float o = sum[C + c];
+            if (tile[c] != at[u] >> 7) {
+              sum[c] += o;
+              tile[c] = at[u] >> 7;
+              o = 0.f;
+            }
+            sum[C + c] = o + a[u][0];
+          } else {
+#pragma unroll
+            for (int c = 0; c < B; ++c) sum[at[u] * BB + c * B + l / NV] += a[u][c];
+          }
+        }
+        __syncwarp();
+      }
+    }
+    for (int x = l; x < here * (B == 1 ? 1 : BB); x += L)
+      __stcs(val + (int64_t(rb) + c0) * BB + x, B == 1 ? sum[x] + sum[C + x] : sum[x]);
+    __syncwarp();  // the sums are the next range's
+  }
+  if constexpr (B > 1) {
+    const int64_t q1 = (unit + 1) * R < n_long ? (unit + 1) * R : n_long;
+    for (int64_t q2 = unit * R; q2 < q1; ++q2) {
+      const int32_t r = ~__ldg(long_rows + q2);
+      if (r < 0) continue;
+      // a lane per value, every incidence of the row looked at
+      const int32_t rp = __ldg(row_ptr + r), words = (__ldg(row_ptr + r + 1) - rp) * BB;
+      for (int x = lane; x < words; x += 32) {
+        const int c = x / BB, c1 = (x % BB) / B, c2 = x % B;
+        float acc = 0.f;
+        for (int32_t t = __ldg(inc_off + r); t < __ldg(inc_off + r + 1); ++t) {
+          const int32_t s = __ldg(inc + t);
+          const float* src = A + int64_t(s / NV) * (N * N) + (c1 * NV + s % NV) * N + c2 * NV;
+#pragma unroll
+          for (int i = 0; i < NV; ++i)
+            if (__ldg(colpos + int64_t(t) * NV + i) == c) acc += __ldg(src + i);
+        }
+        val[int64_t(rp) * BB + x] = acc;
+      }
+    }
+  }
+}
+
+struct BlockParams {
+  const int32_t *inc_off, *inc;
+  const uint8_t* colpos;
+  const int32_t *row_ptr, *order, *blk_off;
+  const int2* slots;
+  const int32_t* long_rows;
+  const RowCounts* counts;
+  const float* A;
+  float* val;
+  int vec_A;
+};
+
+// The blocks block(0), block(1), .. below nblk of a kind that a warp serves;
+// sm: its shared memory, whose sums are zero before and after.
+template <int NV, int B, int KIND, class Blocks>
+__device__ __forceinline__ void assemble_block_rows(const BlockParams& p, const Blocks& block, int64_t nblk,
+                                                    unsigned char* sm, int lane) {
+  using BP = BlockPlan<B>;
+  using K = BlockRows<B, KIND>;
+  constexpr int BB = B * B, G = K::rows, N = NV * B, U = BP::batch;
+  constexpr uint32_t kPad = pad_word(K::cols), kCols = 0x3Fu << K::shift;
+  constexpr int kPart = int(BP::sums);  // from a sum to the open tile sum
+  char* mine = reinterpret_cast<char*>(sm) + 4 * lane;
+  char* stage = reinterpret_cast<char*>(sm) + BP::stage_off + 16 * lane;
+  const int g = lane / BB, q = lane % BB;  // row of the block, component (c, c2) = (q / B, q % B)
+  // offset of the component's row and columns in A_e, without the element slot
+  const float* Aq = p.A + (B == 1 ? 0 : (q / B) * NV * N + (q % B) * NV);
+  const int32_t* order = p.order;  // of block 0 of the kind's numbering
+  if (KIND == ROW_SHORT)
+    order += int64_t(p.counts->wide_blocks()) * (kWideRows - G);
+  // A block's first and last unit of slots and the lane's row in it; then that
+  // row's bounds and the slots of the first batch.  Both are loaded ahead (two
+  // blocks and one), for the latency of these loads is that of a short block's sums.
+  struct Head {
+    int32_t row, s0, s1;
+  };
+  auto load_head = [&](int64_t at) {
+    Head h{-1, 0, 0};
+    if (at < nblk) {
+      h.s0 = __ldg(p.blk_off + at);
+      h.s1 = __ldg(p.blk_off + at + 1);
+      if (g < G) h.row = __ldg(order + at * G + g);
+    }
+    return h;
+  };
+  int2 ahead[U];  // slots of the next batch to load
+  auto load_slots = [&](const Head& h, int k0) {
+    const int2* sl = p.slots + int64_t(h.s0) * K::unit + g;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool on = g < G && (k0 + u) * K::units < h.s1 - h.s0;
+      ahead[u] = on ? __ldg(sl + int64_t(k0 + u) * G) : make_int2(-1, int(kPad));
+    }
+  };
+  int32_t rb = 0, re = 0;
+  auto load_row = [&](const Head& h) {
+    rb = h.row >= 0 ? __ldg(p.row_ptr + h.row) : 0;
+    re = h.row >= 0 ? __ldg(p.row_ptr + h.row + 1) : 0;
+  };
+  Head cur = load_head(block(0)), next = load_head(block(1));
+  load_row(cur);
+  load_slots(cur, 0);
+  for (int i = 0; block(i) < nblk; ++i) {
+    const Head next2 = load_head(block(i + 2));
+    const int steps = (cur.s1 - cur.s0) / K::units;
+    // row (c, i) of A_e, columns (c2, 0 .. NV-1): for tets 16 bytes at a multiple of 16
+    auto piece = [&](int32_t s) {
+      return B == 1 ? int64_t(s) * NV : int64_t(s / NV) * (N * N) + (s % NV) * N;
+    };
+    // adds a step's piece; its NV columns differ (or are all the pad column): read all, add, write all
+    auto add_step = [&](const float(&a)[4], uint32_t w) {
+      char* at[NV];
+      float s[NV], o[NV];
+#pragma unroll
+      for (int j = 0; j < NV; ++j) at[j] = mine + ((j == 0 ? w << K::shift : w >> (8 * j - K::shift)) & kCols);
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        s[j] = *reinterpret_cast<float*>(at[j]);
+        if (B == 1) o[j] = *reinterpret_cast<float*>(at[j] + kPart);
+      }
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        if constexpr (B == 1) {
+          const bool first = w & (kFirst << (8 * j)), last = w & (kLast << (8 * j));
+          float r = (first ? 0.f : o[j]) + a[j];
+          if (last) r = s[j] + r;
+          *reinterpret_cast<float*>(at[j] + (last ? 0 : kPart)) = r;
+        } else {
+          *reinterpret_cast<float*>(at[j]) = s[j] + a[j];
+        }
+      }
+    };
+    if constexpr (BP::staged) {
+      constexpr int T = BP::stages;
+      uint32_t word[T][U];  // column words of the batches in flight
+      auto copy_batch = [&](int st) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          copy_piece<NV>(stage + (st * U + u) * 512, Aq, piece(ahead[u].x), ahead[u].x >= 0, p.vec_A);
+          word[st][u] = uint32_t(ahead[u].y);
+        }
+        cp_async_commit();
+      };
+#pragma unroll
+      for (int st = 0; st < T - 1; ++st) {
+        copy_batch(st);
+        load_slots(cur, (st + 1) * U);
+      }
+      for (int k0 = 0; k0 < steps; k0 += T * U)
+#pragma unroll
+        for (int st = 0; st < T; ++st) {  // the batch at k0 + st * U, in stage st
+          copy_batch(st == 0 ? T - 1 : st - 1);
+          load_slots(cur, k0 + (st + T) * U);
+          cp_async_wait<T - 1>();
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float4 v = *reinterpret_cast<const float4*>(stage + (st * U + u) * 512);
+            add_step({v.x, v.y, v.z, v.w}, word[st][u]);
+          }
+        }
+      cp_async_wait<0>();
+    } else {
+      for (int k0 = 0; k0 < steps; k0 += U) {
+        float a[U][4];
+        uint32_t word[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float* src = Aq + piece(ahead[u].x);
+          word[u] = uint32_t(ahead[u].y);
+#pragma unroll
+          for (int j = 0; j < NV; ++j) a[u][j] = 0.f;
+          if (ahead[u].x >= 0) {
+            if (NV == 4 && p.vec_A) {
+              const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+              a[u][0] = v.x, a[u][1] = v.y, a[u][2] = v.z, a[u][3] = v.w;
+            } else {
+#pragma unroll
+              for (int j = 0; j < NV; ++j) a[u][j] = __ldg(src + j);
+            }
+          }
+        }
+        load_slots(cur, k0 + U);
+#pragma unroll
+        for (int u = 0; u < U; ++u) add_step(a[u], word[u]);
+      }
+    }
+    const int32_t row0 = rb;
+    const int len = re - rb;
+    load_row(next);
+    load_slots(next, 0);
+    const int maxlen = __reduce_max_sync(0xffffffffu, len);
+    if constexpr (B == 1) {
+      // pack the rows' values where the open tile sums were (all closed) and
+      // store them coalesced: as one run where the rows are neighbours, else
+      // row by row, two at a time where they are short
+      int off = len;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, off, d);
+        if (lane >= d) off += up;
+      }
+      const int total = __shfl_sync(0xffffffffu, off, 31);
+      off -= len;
+      __syncwarp();
+      float* pack = reinterpret_cast<float*>(sm + kPart);
+      for (int c = 0; c < maxlen; ++c)
+        if (c < len) {
+          float* w = reinterpret_cast<float*>(mine + (c << K::shift));
+          pack[off + c] = *w;
+          *w = 0.f;
+        }
+      __syncwarp();
+      const int32_t run = __shfl_sync(0xffffffffu, row0, 0);  // every block has a first row
+      if (__all_sync(0xffffffffu, len == 0 || row0 - off == run)) {
+        for (int x = lane; x < total; x += 32) __stcs(p.val + int64_t(run) + x, pack[x]);
+      } else {
+        const int place = off << 6 | len;  // within the pack: at most 1024 values, 63 of a row
+        auto store = [&](int row, int c) {
+          const int32_t to = __shfl_sync(0xffffffffu, row0, row);
+          const int from = __shfl_sync(0xffffffffu, place, row), m = from & 63;
+          const float* src = pack + (from >> 6);
+          if (c < m) __stcs(p.val + int64_t(to) + c, src[c]);
+          if (KIND == ROW_WIDE && c + 32 < m) __stcs(p.val + int64_t(to) + c + 32, src[c + 32]);
+        };
+        if (KIND == ROW_SHORT && maxlen <= 16) {
+#pragma unroll 4
+          for (int h = 0; h < G; h += 2) store(h + (lane >> 4), lane & 15);
+        } else {
+#pragma unroll 4
+          for (int h = 0; h < G; ++h) store(h, lane);
+        }
+      }
+    } else {
+      // a lane's values straight from its bank: 36 (16) contiguous bytes per row and column
+      float* out = p.val + int64_t(row0) * BB + q;
+      for (int c = 0; c < maxlen; ++c)
+        if (c < len) {
+          float* w = reinterpret_cast<float*>(mine + (c << K::shift));
+          out[c * BB] = *w;
+          *w = 0.f;
+        }
+    }
+    __syncwarp();  // the sums are the next block's
+    cur = next;
+    next = next2;
+  }
+}
+
 // One warp per row block: 32 rows of a scalar form, 8 of 2 x 2 blocks, 3 of
 // 3 x 3 blocks; lane g * B^2 + q serves component q of row g.  A row kernel
 // and not a tile pass with records per entry, because its traffic is one read
@@ -303,195 +786,59 @@ __device__ __forceinline__ void copy_piece(void* dst, const float* A, int64_t of
 // 5.5 warps per SM) -> 149 us, 4.8 TB/s of the bytes it cannot do without.
 // What bounds it: the L1 and shared-memory pipe (two or three conflict-free
 // accesses a contribution, and a tag look-up per element row).
+// The long rows come first, then the wide ones: they take longest.
 template <int NV, int B>
 __global__ void __launch_bounds__(BlockPlan<B>::warps * 32, BlockPlan<B>::min_ctas)
-    assemble_blocks_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
-                           const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                           const int32_t* blk_off, const int2* __restrict__ slots, int64_t slot_cap,
-                           const float* __restrict__ A, int64_t n_vert, float* __restrict__ val, int vec_A) {
+    assemble_blocks_kernel(const __grid_constant__ BlockParams p) {
   using BP = BlockPlan<B>;
-  constexpr int BB = B * B, G = block_rows(B), N = NV * B, U = BP::batch;
   extern __shared__ __align__(128) unsigned char block_sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* wbase = block_sm + size_t(warp) * BP::per_warp;
-  float* tot = reinterpret_cast<float*>(wbase);
-  char* mine = reinterpret_cast<char*>(wbase) + 4 * lane;
-  char* stage = reinterpret_cast<char*>(wbase) + BP::stage_off + 16 * lane;
-  constexpr int kPart = int(BP::sums);     // from a sum to the open tile sum
-  const int g = lane / BB, q = lane % BB;  // row of the block, component (c, c2) = (q / B, q % B)
-  // offset of the component's row and columns in A_e, without the element slot
-  const float* Aq = A + (B == 1 ? 0 : (q / B) * NV * N + (q % B) * NV);
-  const int64_t nblk = (n_vert + G - 1) / G;
+  unsigned char* sm = block_sm + size_t(warp) * BP::per_warp;
+  const int64_t S = int64_t(gridDim.x) * BP::warps;
   int64_t b = int64_t(blockIdx.x) * BP::warps + warp;
-  grid_wait(b, blk_off);
-  const bool room = int64_t(blk_off[nblk]) * G <= slot_cap;
+  const RowCounts* counts = p.counts;
+  grid_wait(b, counts);
+  const int n_long = counts->n_long;
+  const int64_t long_units = (int64_t(n_long) + LongPlan<NV, B>::rows - 1) / LongPlan<NV, B>::rows;
+  for (; b < long_units; b += S)
+    assemble_long_rows<NV, B>(p.inc_off, p.inc, p.colpos, p.row_ptr, p.long_rows, n_long, b, p.A, p.val,
+                              reinterpret_cast<float*>(sm), lane);
+  b -= long_units;
   // the sums are zero at the start of every block: zeroed here, and again as they are read out
-  for (int c = 0; c <= kFastCols; ++c) *reinterpret_cast<float*>(mine + c * 128) = 0.f;
-  // a lane per value, every incidence of the row looked at
-  auto scan_row = [&](int64_t r) {
-    const int32_t rp = __ldg(row_ptr + r), t0 = __ldg(inc_off + r), t1 = __ldg(inc_off + r + 1);
-    const int words = (__ldg(row_ptr + r + 1) - rp) * BB;
-    for (int x = lane; x < words; x += 32) {
-      const int c = x / BB, c1 = (x % BB) / B, c2 = x % B;
-      float sum = 0.f, part = 0.f;
-      int tile = -1;
-      for (int32_t t = t0; t < t1; ++t) {
-        const int32_t s = __ldg(inc + t);
-        const float* src = A + int64_t(s / NV) * (N * N) + (c1 * NV + s % NV) * N + c2 * NV;
-        if (B == 1 && (s / NV) >> 5 != tile) {
-          sum += part;
-          part = 0.f;
-          tile = (s / NV) >> 5;
-        }
-#pragma unroll
-        for (int j = 0; j < NV; ++j)
-          if (__ldg(colpos + int64_t(t) * NV + j) == c) (B == 1 ? part : sum) += __ldg(src + j);
-      }
-      val[int64_t(rp) * BB + x] = sum + part;
-    }
-  };
-  for (; b < nblk; b += int64_t(gridDim.x) * BP::warps) {
-    const int64_t r0 = b * G;
-    const int nr = int(n_vert - r0 < G ? n_vert - r0 : G);
-    const int32_t s0 = __ldg(blk_off + b), steps = __ldg(blk_off + b + 1) - s0;
-    const int32_t rp0 = __ldg(row_ptr + r0), total = __ldg(row_ptr + r0 + nr) - rp0;
-    if (total == 0) continue;
-    if (room && steps > 0) {
-      const bool live = g < nr;
-      const int32_t rb = live ? __ldg(row_ptr + r0 + g) : 0;
-      const int row_len = live ? __ldg(row_ptr + r0 + g + 1) - rb : 0;
-      // scalar forms: a long row's slots are padding, it is scanned below
-      const uint32_t long_lanes = B == 1 ? __ballot_sync(0xffffffffu, row_len > kFastCols) : 0u;
-      const int len = B == 1 && row_len > kFastCols ? 0 : row_len;
-      const int2* sl = slots + int64_t(s0) * G + g;
-      int2 ahead[U];  // slots of the next batch to load
-      auto load_slots = [&](int k0) {
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          ahead[u] = live && k0 + u < steps ? __ldg(sl + (k0 + u) * G) : make_int2(-1, kPadCol * 0x01010101);
-      };
-      // row (c, i) of A_e, columns (c2, 0 .. NV-1): for tets 16 bytes at a multiple of 16
-      auto piece = [&](int32_t s) {
-        return B == 1 ? int64_t(s) * NV : int64_t(s / NV) * (N * N) + (s % NV) * N;
-      };
-      // adds a step's piece; its NV columns differ (or are all the pad column): read all, add, write all
-      auto add_step = [&](const float(&a)[4], uint32_t w) {
-        char* at[NV];
-        float s[NV], o[NV];
-#pragma unroll
-        for (int j = 0; j < NV; ++j) at[j] = mine + ((j == 0 ? w << 7 : w >> (8 * j - 7)) & (0x3Fu << 7));
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-          s[j] = *reinterpret_cast<float*>(at[j]);
-          if (B == 1) o[j] = *reinterpret_cast<float*>(at[j] + kPart);
-        }
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-          if constexpr (B == 1) {
-            const bool first = w & (kFirst << (8 * j)), last = w & (kLast << (8 * j));
-            float r = (first ? 0.f : o[j]) + a[j];
-            if (last) r = s[j] + r;
-            *reinterpret_cast<float*>(at[j] + (last ? 0 : kPart)) = r;
-          } else {
-            *reinterpret_cast<float*>(at[j]) = s[j] + a[j];
-          }
-        }
-      };
-      load_slots(0);
-      if constexpr (BP::staged) {
-        constexpr int S = BP::stages;
-        uint32_t word[S][U];  // column words of the batches in flight
-        auto copy_batch = [&](int st) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            copy_piece<NV>(stage + (st * U + u) * 512, Aq, piece(ahead[u].x), ahead[u].x >= 0, vec_A);
-            word[st][u] = uint32_t(ahead[u].y);
-          }
-          cp_async_commit();
-        };
-#pragma unroll
-        for (int st = 0; st < S - 1; ++st) {
-          copy_batch(st);
-          load_slots((st + 1) * U);
-        }
-        for (int k0 = 0; k0 < steps; k0 += S * U)
-#pragma unroll
-          for (int st = 0; st < S; ++st) {  // the batch at k0 + st * U, in stage st
-            copy_batch(st == 0 ? S - 1 : st - 1);
-            load_slots(k0 + (st + S) * U);
-            cp_async_wait<S - 1>();
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const float4 v = *reinterpret_cast<const float4*>(stage + (st * U + u) * 512);
-              add_step({v.x, v.y, v.z, v.w}, word[st][u]);
-            }
-          }
-        cp_async_wait<0>();
-      } else {
-        for (int k0 = 0; k0 < steps; k0 += U) {
-          float a[U][4];
-          uint32_t word[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const float* src = Aq + piece(ahead[u].x);
-            word[u] = uint32_t(ahead[u].y);
-#pragma unroll
-            for (int j = 0; j < NV; ++j) a[u][j] = 0.f;
-            if (ahead[u].x >= 0) {
-              if (NV == 4 && vec_A) {
-                const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
-                a[u][0] = v.x, a[u][1] = v.y, a[u][2] = v.z, a[u][3] = v.w;
-              } else {
-#pragma unroll
-                for (int j = 0; j < NV; ++j) a[u][j] = __ldg(src + j);
-              }
-            }
-          }
-          load_slots(k0 + U);
-#pragma unroll
-          for (int u = 0; u < U; ++u) add_step(a[u], word[u]);
-        }
-      }
-      const int maxlen = __reduce_max_sync(0xffffffffu, len);
-      if (B == 1 && long_lanes == 0) {
-        // pack the rows' values where the open tile sums were (all closed) and store them coalesced
-        __syncwarp();
-        float* pack = reinterpret_cast<float*>(wbase + kPart);
-        for (int c = 0; c < maxlen; ++c)
-          if (c < len) {
-            float* w = reinterpret_cast<float*>(mine + c * 128);
-            pack[rb - rp0 + c] = *w;
-            *w = 0.f;
-          }
-        __syncwarp();
-        for (int x = lane; x < total; x += 32) __stcs(val + int64_t(rp0) + x, pack[x]);
-      } else {
-        // a lane's values straight from its bank: 36 (16) contiguous bytes per row and column
-        float* out = val + int64_t(rb) * BB + q;
-        for (int c = 0; c < maxlen; ++c)
-          if (c < len) {
-            float* w = reinterpret_cast<float*>(mine + c * 128);
-            out[c * BB] = *w;
-            *w = 0.f;
-          }
-      }
-      __syncwarp();  // the sums are the next block's
-      if constexpr (B == 1)
-        for (uint32_t left = long_lanes; left; left &= left - 1) scan_row(r0 + __ffs(left) - 1);
-    } else {
-      for (int h = 0; h < nr; ++h) scan_row(r0 + h);
+  for (int x = lane; x < int(BP::stage_off / 4); x += 32) reinterpret_cast<float*>(sm)[x] = 0.f;
+  __syncwarp();
+  const int64_t nblk = counts->template blocks<B>(), wide = counts->wide_blocks();
+  int64_t more = 0, lead = 0, mine = 0;
+  if constexpr (B == 1) {
+    if (wide > 0) {
+      if (b < wide)
+        assemble_block_rows<NV, B, ROW_WIDE>(p, [=](int i) { return b + i * S; }, wide, sm, lane);
+      // Warps below more have taken a wide block more than the others, which
+      // have a lead of as many short blocks as make up its steps.
+      more = wide % S;
+      const int64_t wide_units = p.blk_off[wide], n_short = nblk - wide;
+      const int64_t fair = 2 * wide_units * n_short / (wide * (p.blk_off[nblk] - wide_units + 1));
+      lead = more == 0 ? 0 : fair * (S - more) < n_short ? fair : n_short / (S - more);
+      mine = b < more ? 0 : lead;
     }
   }
+  auto block = [=](int i) {
+    return i < mine ? wide + (b - more) + i * (S - more) : wide + lead * (S - more) + b + (i - mine) * S;
+  };
+  assemble_block_rows<NV, B, ROW_SHORT>(p, block, nblk, sm, lane);
 }
 
 struct AsmLayout {
   int32_t *inc_off, *inc, *row_ptr, *col_idx, *cursor, *partials;
-  int32_t* flag;  // [0] build flags, [1] tile records (scalar forms)
+  int32_t* flag;  // [0] build flags, [1] tile records (scalar forms), an element repeats a vertex (blocks)
+  int32_t* near;    // row_near_kernel's counts
+  RowCounts* counts;
   uint8_t* colpos;
   // row blocks (P1 forms and elasticity)
-  int32_t* blk_off;  // [blocks + 1] first step of each block
-  int2* slots;       // [steps][block_rows]: (element slot or -1, column word)
-  int64_t slot_cap;
+  int32_t* order;      // the rows of every block, the wide blocks first: the row, or -1
+  int32_t* blk_off;    // [blocks + 1] first slot of each block, in units
+  int2* slots;         // of every block, [steps][rows]: (element slot or -1, column word)
+  int32_t* long_rows;  // [n_long]
   size_t bytes;
 };
 
@@ -507,20 +854,29 @@ AsmLayout asm_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
     return o;
   };
   AsmLayout L{};
-  // Room for padding the rows of a block to its longest one: twice the
-  // incidences (a cube's rows need 1.1 times; a mesh that needs more than
-  // twice takes the scanning path of the kernel, which reads no slots).
-  L.slot_cap = 2 * n_elem * nv + 1024;
+  // Room for the padded slots of every mesh: a window in row order takes 1.5
+  // times its incidences, a sorted one as many as its incidences and, for its
+  // first block, the largest count for every row (block_order_kernel).  A
+  // window of short rows and one of wide rows pad the same per row.
+  const int64_t n_inc = n_elem * nv, n_rows = n_vert < n_inc ? n_vert : n_inc;
+  const int64_t first_blocks = (n_rows / BlockRows<1, ROW_SHORT>::win_rows + 2) * max_incidences(int(nv));
+  const int64_t slot_cap = n_inc + n_inc / 2 + 32 * (first_blocks < n_inc ? first_blocks : n_inc);
+  // and, before the slots, for the flags, their scan and the rows (launch_row_blocks)
+  const int64_t n_keys = n_vert > n_inc ? n_vert : n_inc;
+  const size_t slot_bytes = sizeof(int2) * size_t(slot_cap);
+  const size_t key_bytes = sizeof(int32_t) * size_t(2 * n_keys + 1 + n_rows);
   const size_t o_inc_off = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_inc = take(sizeof(int32_t) * size_t(n_elem * nv));
   const size_t o_colpos = take(size_t(cap));
   const size_t o_row_ptr = take(sizeof(int32_t) * size_t(n_vert + 1));
   const size_t o_col = take(sizeof(int32_t) * size_t(cap));  // capacity: every entry distinct
-  const size_t o_cursor = take(sizeof(int32_t) * size_t(n_vert + 1));
-  const size_t o_part = take(sizeof(int32_t) * scan_partials_count(n_vert + 1));
-  const size_t o_flag = take(sizeof(int32_t) * 4);
-  const size_t o_blk = take(sizeof(int32_t) * size_t(n_vert + 2));
-  const size_t o_slots = take(sizeof(int2) * size_t(L.slot_cap));
+  const size_t o_cursor = take(sizeof(int32_t) * size_t(n_vert + 4));
+  const size_t o_part = take(sizeof(int32_t) * scan_partials_count(n_keys + 1));
+  const size_t o_flag = take(sizeof(int32_t) * 8);
+  const size_t o_order = take(sizeof(int32_t) * size_t(n_vert + 64));
+  const size_t o_blk = take(sizeof(int32_t) * size_t(n_vert + 4));
+  const size_t o_slots = take(slot_bytes > key_bytes ? slot_bytes : key_bytes);
+  const size_t o_long = take(sizeof(int32_t) * size_t(n_vert));
   char* b = static_cast<char*>(base);
   L.inc_off = reinterpret_cast<int32_t*>(b + o_inc_off);
   L.inc = reinterpret_cast<int32_t*>(b + o_inc);
@@ -530,8 +886,12 @@ AsmLayout asm_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
   L.cursor = reinterpret_cast<int32_t*>(b + o_cursor);
   L.partials = reinterpret_cast<int32_t*>(b + o_part);
   L.flag = reinterpret_cast<int32_t*>(b + o_flag);
+  L.near = L.flag + 2;
+  L.counts = reinterpret_cast<RowCounts*>(L.flag + 4);
+  L.order = reinterpret_cast<int32_t*>(b + o_order);
   L.blk_off = reinterpret_cast<int32_t*>(b + o_blk);
   L.slots = reinterpret_cast<int2*>(b + o_slots);
+  L.long_rows = reinterpret_cast<int32_t*>(b + o_long);
   L.bytes = off;
   return L;
 }
@@ -555,31 +915,92 @@ cudaError_t launch_pattern(int dim, const int32_t* conn, int64_t n_vert, const A
   return cudaGetLastError();
 }
 
-// The row blocks of a built pattern (B = block size of the form).  Scalar
-// forms also count their tile records into L.flag[1].
-template <int NV, int B>
-cudaError_t launch_row_blocks(int64_t n_vert, const AsmLayout& L, cudaStream_t st) {
-  const int64_t nblk = (n_vert + block_rows(B) - 1) / block_rows(B);
-  block_steps_kernel<NV, B><<<grid_of(nblk, 256), 256, 0, st>>>(L.inc_off, L.row_ptr, L.colpos, n_vert, L.cursor);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_exclusive_scan(L.cursor, nblk, L.partials, L.blk_off, st);
+// The rows of a kind in order, into rows, and their number.
+template <int NV, int B, int KIND>
+cudaError_t launch_rows_of(int64_t n_keys, int by_number, int repeats, int64_t n_vert, const AsmLayout& L,
+                           int32_t* rows, int32_t* n_rows, cudaStream_t st) {
+  // flags by key and their scan use the room of the slots
+  int32_t* flag = reinterpret_cast<int32_t*>(L.slots);
+  int32_t* foff = flag + n_keys;
+  const unsigned gv = grid_of(n_vert, 256);
+  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int32_t) * size_t(n_keys), st);
   if (e != cudaSuccess) return e;
-  block_fill_kernel<NV, B><<<grid_of(n_vert, 256), 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off,
-                                                                 n_vert, L.slot_cap, L.slots, L.flag + 1);
+  row_flag_kernel<NV, B, KIND><<<gv, 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.row_ptr, by_number, repeats, n_vert,
+                                                flag);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_exclusive_scan(flag, n_keys, L.partials, foff, st);
+  if (e != cudaSuccess) return e;
+  row_place_kernel<NV, B, KIND><<<gv, 256, 0, st>>>(L.inc_off, L.inc, L.colpos, foff, by_number, repeats, n_vert,
+                                                 rows);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(n_rows, foff + n_keys, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+  return e;
+}
+
+// The row blocks of a built pattern (B = block size of the form), the rows by
+// their number or by their first incidence.  Scalar forms also count their
+// tile records into L.flag[1].
+template <int NV, int B>
+cudaError_t launch_row_blocks(int64_t n_elem, int64_t n_vert, int by_number, int repeats, const AsmLayout& L,
+                              cudaStream_t st) {
+  const int64_t n_keys = by_number ? n_vert : n_elem * NV;
+  const int64_t cap = n_vert / BlockRows<B, ROW_SHORT>::unit + 2;  // blocks at most
+  const unsigned gv = grid_of(n_vert, 256);
+  int32_t* rows = reinterpret_cast<int32_t*>(L.slots) + 2 * n_keys + 1;  // behind the flags and their scan
+  cudaError_t e = launch_rows_of<NV, B, ROW_LONG>(n_keys, by_number, repeats, n_vert, L, L.long_rows,
+                                                  &L.counts->n_long, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.cursor, 0, sizeof(int32_t) * size_t(cap), st);
+  if constexpr (B == 1) {
+    if (e == cudaSuccess)
+      e = launch_rows_of<NV, B, ROW_WIDE>(n_keys, by_number, 0, n_vert, L, rows, &L.counts->n_wide, st);
+    if (e != cudaSuccess) return e;
+    block_order_kernel<NV, B, ROW_WIDE><<<grid_of(n_vert, BlockRows<B, ROW_WIDE>::win_rows), 256, 0, st>>>(
+        L.inc_off, rows, L.counts, L.order, L.cursor);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess)
+    e = launch_rows_of<NV, B, ROW_SHORT>(n_keys, by_number, repeats, n_vert, L, rows, &L.counts->n_short, st);
+  if (e != cudaSuccess) return e;
+  block_order_kernel<NV, B, ROW_SHORT><<<grid_of(n_vert, BlockRows<B, ROW_SHORT>::win_rows), 256, 0, st>>>(
+      L.inc_off, rows, L.counts, L.order, L.cursor);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_exclusive_scan(L.cursor, cap, L.partials, L.blk_off, st);
+  if (e != cudaSuccess) return e;
+  if constexpr (B == 1)
+    block_fill_kernel<NV, B, ROW_WIDE><<<gv, 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.order, L.blk_off, L.long_rows,
+                                                           L.counts, L.slots, L.flag + 1);
+  block_fill_kernel<NV, B, ROW_SHORT><<<gv, 256, 0, st>>>(L.inc_off, L.inc, L.colpos, L.order, L.blk_off, L.long_rows,
+                                                          L.counts, L.slots, L.flag + 1);
   return cudaGetLastError();
 }
 
 template <int NV, int B>
-cudaError_t launch_assemble_t(const AsmLayout& L, const float* A, int64_t n_vert, float* val, cudaStream_t st) {
+cudaError_t launch_assemble_t(const AsmLayout& L, const float* A, int64_t n_elem, int64_t n_vert, float* val,
+                              cudaStream_t st) {
   auto kern = assemble_blocks_kernel<NV, B>;
   constexpr int warps = BlockPlan<B>::warps;
   constexpr size_t smem = BlockPlan<B>::smem;
   const cudaError_t e = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  const int64_t nblk = (n_vert + block_rows(B) - 1) / block_rows(B);
-  const unsigned g = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, nblk * 32, 0);
-  return launch_chained(kern, g, unsigned(warps * 32), smem, st, L.inc_off, L.inc, L.colpos, L.row_ptr, L.blk_off,
-                        L.slots, L.slot_cap, A, n_vert, val, int(reinterpret_cast<uintptr_t>(A) % 16 == 0));
+  // blocks, and units of long rows: a row of more than cols columns has cols / (NV - 1) elements or more
+  constexpr int cols = BlockRows<B, B == 1 ? ROW_WIDE : ROW_SHORT>::cols;
+  const int64_t units = n_vert / BlockRows<B, ROW_SHORT>::rows + 2 +
+                        n_elem * NV * (NV - 1) / cols / LongPlan<NV, B>::rows;
+  // On triangles an element row's 12 bytes pass through L1, three copies to a
+  // line that must stay until the third: 16 CTAs an SM leave L1 room for them,
+  // the 19 that fit leave too little (barycentric 600^2 square 112 -> 80 us,
+  // 900^2 square 60 -> 54, numbered at random 78 -> 68; 14 CTAs 82, 56, 68).
+  constexpr int ctas = BlockPlan<B>::staged && NV == 3 ? 16 : 0;
+  if (ctas > 0) {
+    const cudaError_t c = cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
+                                               cudaFuncAttributePreferredSharedMemoryCarveout,
+                                               int((ctas * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024)));
+    if (c != cudaSuccess) return c;
+  }
+  const unsigned g = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, units * 32, ctas);
+  const BlockParams p{L.inc_off, L.inc, L.colpos, L.row_ptr, L.order, L.blk_off, L.slots, L.long_rows, L.counts, A, val,
+                      int(reinterpret_cast<uintptr_t>(A) % 16 == 0)};
+  return launch_chained(kern, g, unsigned(warps * 32), smem, st, p);
 }
 
 // ------------------------------------------------------------------ P2 unknowns (vertices, then edges)
@@ -1074,7 +1495,7 @@ fem_status fem_assembly_build(const fem_mesh* mesh, int32_t form, void* ws, size
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int nv = mesh->dim + 1;
   const int64_t V = mesh->n_vert;
-  cudaError_t e = cudaMemsetAsync(L.flag, 0, sizeof(int32_t) * 4, st);
+  cudaError_t e = cudaMemsetAsync(L.flag, 0, sizeof(int32_t) * 8, st);
   if (e == cudaSuccess && mesh->n_elem > 0) {
     fem::check_conn_kernel<<<fem::grid_of(mesh->n_elem * nv, 256), 256, 0, st>>>(mesh->conn, mesh->n_elem * nv, V,
                                                                                   L.flag);
@@ -1086,24 +1507,33 @@ fem_status fem_assembly_build(const fem_mesh* mesh, int32_t form, void* ws, size
   if (e == cudaSuccess) e = fem::launch_exclusive_scan(L.cursor, V, L.partials, L.row_ptr, st);
   if (e == cudaSuccess && V > 0) e = fem::launch_pattern<true>(mesh->dim, mesh->conn, V, L, st);
   const int B = asm_block(form, mesh->dim);
-  if (e == cudaSuccess && B == 1 && mesh->n_elem > 0) {  // the scalar forms refuse an element repeating a vertex
+  if (e == cudaSuccess && mesh->n_elem > 0) {  // the scalar forms refuse an element repeating a vertex
     const unsigned g = fem::grid_of(mesh->n_elem, 256);
+    int32_t* flag = B == 1 ? L.flag : L.flag + 1;
     if (mesh->dim == 2)
-      fem::check_repeat_kernel<3><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, L.flag);
+      fem::check_repeat_kernel<3><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, flag);
     else
-      fem::check_repeat_kernel<4><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, L.flag);
+      fem::check_repeat_kernel<4><<<g, 256, 0, st>>>(mesh->conn, mesh->n_elem, flag);
     e = cudaGetLastError();
   }
-  int32_t host[2] = {0, 0}, nrec = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&host[0], L.flag, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&host[1], L.row_ptr + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && V > 0) {
+    fem::row_near_kernel<<<fem::grid_of(V, 256), 256, 0, st>>>(L.inc_off, L.inc, V, L.near);
+    e = cudaGetLastError();
+  }
+  int32_t host[4] = {0, 0, 0, 0}, nz = 0, nrec = 0;  // build flags, repeated vertices (blocks), near
+  if (e == cudaSuccess) e = cudaMemcpyAsync(host, L.flag, sizeof(host), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&nz, L.row_ptr + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && host[0] == 0 && V > 0) {
+  if (e == cudaSuccess && host[0] == 0 && V > 0 && mesh->n_elem > 0) {
+    const int by_number = 2 * int64_t(host[3]) >= host[2], repeats = host[1] != 0;
     if (mesh->dim == 2)
-      e = B == 1 ? fem::launch_row_blocks<3, 1>(V, L, st) : fem::launch_row_blocks<3, 2>(V, L, st);
+      e = B == 1 ? fem::launch_row_blocks<3, 1>(mesh->n_elem, V, by_number, repeats, L, st)
+                 : fem::launch_row_blocks<3, 2>(mesh->n_elem, V, by_number, repeats, L, st);
     else
-      e = B == 1 ? fem::launch_row_blocks<4, 1>(V, L, st) : fem::launch_row_blocks<4, 3>(V, L, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nrec, L.flag + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+      e = B == 1 ? fem::launch_row_blocks<4, 1>(mesh->n_elem, V, by_number, repeats, L, st)
+                 : fem::launch_row_blocks<4, 3>(mesh->n_elem, V, by_number, repeats, L, st);
+    if (e == cudaSuccess && B == 1)
+      e = cudaMemcpyAsync(&nrec, L.flag + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
   if (e != cudaSuccess) {
@@ -1114,7 +1544,7 @@ fem_status fem_assembly_build(const fem_mesh* mesh, int32_t form, void* ws, size
   if (host[0] & fem::ASM_ROW_TOO_LONG)
     return asm_fail(FEM_ERR_UNSUPPORTED, "a vertex has more than 128 incident elements or 255 neighbours");
   if (host[0] & fem::ASM_REPEATED_VERTEX) return asm_fail(FEM_ERR_UNSUPPORTED, "an element repeats a vertex");
-  if (nnz) *nnz = host[1];
+  if (nnz) *nnz = nz;
   if (n_records) *n_records = nrec;
   return FEM_OK;
 }
@@ -1181,11 +1611,11 @@ fem_status fem_assemble(const fem_mesh* mesh, int32_t form, const float* A, cons
   } else if (mesh->n_elem == 0) {
     return FEM_OK;
   } else if (mesh->dim == 2) {
-    e = B == 1 ? fem::launch_assemble_t<3, 1>(L, A, mesh->n_vert, values, st)
-               : fem::launch_assemble_t<3, 2>(L, A, mesh->n_vert, values, st);
+    e = B == 1 ? fem::launch_assemble_t<3, 1>(L, A, mesh->n_elem, mesh->n_vert, values, st)
+               : fem::launch_assemble_t<3, 2>(L, A, mesh->n_elem, mesh->n_vert, values, st);
   } else {
-    e = B == 1 ? fem::launch_assemble_t<4, 1>(L, A, mesh->n_vert, values, st)
-               : fem::launch_assemble_t<4, 3>(L, A, mesh->n_vert, values, st);
+    e = B == 1 ? fem::launch_assemble_t<4, 1>(L, A, mesh->n_elem, mesh->n_vert, values, st)
+               : fem::launch_assemble_t<4, 3>(L, A, mesh->n_elem, mesh->n_vert, values, st);
   }
   if (e != cudaSuccess) {
     fem::set_last_error("fem_assemble: %s", cudaGetErrorString(e));
