@@ -1014,6 +1014,23 @@ cudaError_t launch_assemble_t(const AsmLayout& L, const float* A, int64_t n_elem
 // then its edges in the local P2 order) form the connectivity of a second
 // pattern, over the V + n_edges unknowns, which the row kernel assembles.
 
+// The rows' incidences in chunks of four: row r holds chunks [choff[r],
+// choff[r+1]).  They lie behind the column indices of the unknowns, over the
+// entries that the pattern did not need and over the vertex graph, and take no
+// room of their own (252 bytes an element on tets otherwise, a third of the
+// workspace).  A mesh whose unknowns hardly share elements has no room there:
+// its incidences are read as they are.
+struct P2Plan {
+  int32_t n_rows;  // V + n_edges
+  int32_t at;      // of the chunks from g2.col_idx on, in 16 bytes
+  int32_t n;       // chunks
+  int32_t fits;
+  // offsets of the element rows in A, (e * n + i) * n; -1 in the padding
+  __device__ int4* slot4(int32_t* col_idx) const { return reinterpret_cast<int4*>(col_idx) + at; }
+  // [chunk][n]: byte u = the column position of the element's unknown j for incidence u
+  __device__ uint32_t* pos4(int32_t* col_idx) const { return reinterpret_cast<uint32_t*>(slot4(col_idx) + n); }
+};
+
 // Arrays of the P2 assembly: the vertex graph's incidences and pattern
 // (positions per incidence), the edge offsets, the element unknowns, and the
 // unknowns' incidences and pattern.
@@ -1022,12 +1039,9 @@ struct AsmP2Layout {
   AsmLayout g2;  // unknowns (same fields over up to V + E * n_edges rows)
   int32_t* eoff;   // [V + 1]
   int32_t* dofs;   // [E][n]
-  int32_t* n_rows; // one word: V + n_edges
-  // the rows' incidences in chunks of four: row r holds chunks [choff[r], choff[r+1])
-  int32_t* choff;   // [rows + 1]
-  int4* slot4;      // offsets of the element rows in A, (e * n + i) * n; -1 in the padding
-  uint32_t* pos4;   // [chunk][n]: byte u = the column position of the element's unknown j for incidence u
-  int64_t chunk_cap;
+  P2Plan* plan;
+  int32_t* choff() const { return g2.cursor; }  // [rows + 1]
+  int64_t room;    // bytes from g2.col_idx to the end of g1 and eoff, which are dead once g2 is built
   int64_t rows_cap;
   size_t bytes;
 };
@@ -1042,43 +1056,27 @@ AsmP2Layout asm_p2_layout(int dim, int64_t n_elem, int64_t n_vert, void* base) {
     return o;
   };
   char* b = static_cast<char*>(base);
-  auto graph = [&](int64_t rows, int64_t per_elem, AsmLayout& G) {
-    const int64_t cap = n_elem * per_elem * per_elem;
-    const size_t o_inc_off = take(sizeof(int32_t) * size_t(rows + 1));
-    const size_t o_inc = take(sizeof(int32_t) * size_t(n_elem * per_elem));
-    const size_t o_colpos = take(size_t(cap));
-    const size_t o_row_ptr = take(sizeof(int32_t) * size_t(rows + 1));
-    const size_t o_col = take(sizeof(int32_t) * size_t(cap));
-    const size_t o_cursor = take(sizeof(int32_t) * size_t(rows + 1));
-    const size_t o_part = take(sizeof(int32_t) * scan_partials_count(rows + 1));
-    G.inc_off = reinterpret_cast<int32_t*>(b + o_inc_off);
-    G.inc = reinterpret_cast<int32_t*>(b + o_inc);
-    G.colpos = reinterpret_cast<uint8_t*>(b + o_colpos);
-    G.row_ptr = reinterpret_cast<int32_t*>(b + o_row_ptr);
-    G.col_idx = reinterpret_cast<int32_t*>(b + o_col);
-    G.cursor = reinterpret_cast<int32_t*>(b + o_cursor);
-    G.partials = reinterpret_cast<int32_t*>(b + o_part);
+  auto words = [&](int64_t n) { return reinterpret_cast<int32_t*>(b + take(sizeof(int32_t) * size_t(n))); };
+  auto graph = [&](int64_t rows, int64_t per_elem, AsmLayout& G) {  // its columns, the last, are taken by the caller
+    G.inc_off = words(rows + 1);
+    G.inc = words(n_elem * per_elem);
+    G.colpos = reinterpret_cast<uint8_t*>(b + take(size_t(n_elem * per_elem * per_elem)));
+    G.row_ptr = words(rows + 1);
+    G.cursor = words(rows + 1);
+    G.partials = words(int64_t(scan_partials_count(rows + 1)));
   };
   AsmP2Layout L{};
-  graph(n_vert, nv, L.g1);
-  graph(rows_cap, n, L.g2);
-  const size_t o_eoff = take(sizeof(int32_t) * size_t(n_vert + 1));
-  const size_t o_dofs = take(sizeof(int32_t) * size_t(n_elem * n));
-  const size_t o_flag = take(sizeof(int32_t) * 8);
-  // 2.9 chunks per tet on a cube; a mesh that needs more room than this (many
-  // unknowns with few elements each) reads the incidences one by one instead
-  L.chunk_cap = n_elem * 9 / 2 + n_vert + 1024;
-  const size_t o_choff = take(sizeof(int32_t) * size_t(rows_cap + 1));
-  const size_t o_slot4 = take(sizeof(int4) * size_t(L.chunk_cap));
-  const size_t o_pos4 = take(sizeof(uint32_t) * size_t(L.chunk_cap * n));
-  L.choff = reinterpret_cast<int32_t*>(b + o_choff);
-  L.slot4 = reinterpret_cast<int4*>(b + o_slot4);
-  L.pos4 = reinterpret_cast<uint32_t*>(b + o_pos4);
-  L.eoff = reinterpret_cast<int32_t*>(b + o_eoff);
-  L.dofs = reinterpret_cast<int32_t*>(b + o_dofs);
-  L.g1.flag = reinterpret_cast<int32_t*>(b + o_flag);
+  L.dofs = words(n_elem * n);
+  L.g1.flag = words(8);
   L.g2.flag = L.g1.flag;
-  L.n_rows = L.g1.flag + 4;
+  L.plan = reinterpret_cast<P2Plan*>(L.g1.flag + 4);
+  graph(rows_cap, n, L.g2);
+  const size_t col = off;
+  L.g2.col_idx = words(n_elem * n * n);
+  graph(n_vert, nv, L.g1);
+  L.g1.col_idx = words(n_elem * nv * nv);
+  L.eoff = words(n_vert + 1);
+  L.room = int64_t(off - col);
   L.rows_cap = rows_cap;
   L.bytes = off;
   return L;
@@ -1148,8 +1146,17 @@ __global__ void edge_dof_kernel(const int32_t* __restrict__ conn, const int32_t*
   }
 }
 
-__global__ void store_rows_kernel(const int32_t* __restrict__ eoff, int64_t n_vert, int32_t* n_rows) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_rows = int32_t(n_vert + eoff[n_vert]);
+__global__ void store_rows_kernel(const int32_t* __restrict__ eoff, int64_t n_vert, P2Plan* plan) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) plan->n_rows = int32_t(n_vert + eoff[n_vert]);
+}
+
+// Where the chunks lie, and whether they fit (room: bytes from the column indices on).
+__global__ void chunk_plan_kernel(const int32_t* row_ptr, const int32_t* choff, int nb, int64_t room, P2Plan* plan) {
+  if (blockIdx.x || threadIdx.x) return;
+  const int64_t at = (int64_t(row_ptr[plan->n_rows]) + 3) / 4, n = choff[plan->n_rows];
+  plan->at = int32_t(at);
+  plan->n = int32_t(n);
+  plan->fits = 16 * at + n * (16 + 4 * nb) <= room;
 }
 
 // Chunks of four incidences per row.
@@ -1161,8 +1168,10 @@ __global__ void chunk_count_kernel(const int32_t* __restrict__ inc_off, int64_t 
 template <int NB>
 __global__ void chunk_fill_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
                                   const uint8_t* __restrict__ colpos, const int32_t* __restrict__ choff,
-                                  int64_t n_rows, int64_t cap, int4* __restrict__ slot4, uint32_t* __restrict__ pos4) {
-  if (choff[n_rows] > cap) return;  // no room: the rows are read one incidence at a time
+                                  const P2Plan* __restrict__ plan, int64_t n_rows, int32_t* col_idx) {
+  if (!plan->fits) return;
+  int4* slot4 = plan->slot4(col_idx);
+  uint32_t* pos4 = plan->pos4(col_idx);
   for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < n_rows; r += int64_t(gridDim.x) * blockDim.x) {
     const int32_t t0 = inc_off[r], n = inc_off[r + 1] - t0;
     for (int k = 0; k < n; k += 4) {
@@ -1220,10 +1229,10 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    store_rows_kernel<<<1, 32, 0, st>>>(L.eoff, n_vert, L.n_rows);
+    store_rows_kernel<<<1, 32, 0, st>>>(L.eoff, n_vert, L.plan);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(rows_host, L.n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(rows_host, &L.plan->n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(flag_host, G1.flag, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess || *flag_host) return e;
@@ -1239,13 +1248,22 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
   if (e == cudaSuccess && R > 0) {
     row_pattern_kernel<NB, true><<<gr, kPatWarps * 32, 0, st>>>(L.dofs, G2.inc_off, G2.inc, R, G2.cursor,
                                                                  G2.row_ptr, G2.col_idx, G2.colpos, G2.flag);
-    chunk_count_kernel<<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, R, G2.cursor);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = launch_exclusive_scan(G2.cursor, R, G2.partials, L.choff, st);
+  // the counts take room of the vertex graph, which is dead, their scan that of the cursors
+  int32_t* counts = G1.inc_off;
   if (e == cudaSuccess && R > 0) {
-    chunk_fill_kernel<NB><<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, G2.inc, G2.colpos, L.choff, R, L.chunk_cap,
-                                                           L.slot4, L.pos4);
+    chunk_count_kernel<<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, R, counts);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = launch_exclusive_scan(counts, R, G2.partials, L.choff(), st);
+  if (e == cudaSuccess) {
+    chunk_plan_kernel<<<1, 32, 0, st>>>(G2.row_ptr, L.choff(), NB, L.room, L.plan);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && R > 0) {
+    chunk_fill_kernel<NB><<<grid_of(R, 256), 256, 0, st>>>(G2.inc_off, G2.inc, G2.colpos, L.choff(), L.plan, R,
+                                                           G2.col_idx);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(nnz_host, G2.row_ptr + R, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
@@ -1267,25 +1285,33 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
 // between lanes and a byte per incidence took two shuffles or loads for every
 // addition, on the pipe that the additions use (shared-memory and load pipe
 // 76% busy).  The next two chunks, of this row group or the next, are loaded
-// under the additions.  61^3 cube: 312 -> 281 us; bound by instruction issue
+// under the additions.  61^3 cube: 312 -> 277 us; bound by instruction issue
 // (68% active) and that pipe (70%), two accesses an addition, 2.6 wavefronts
-// each over the random columns of three rows.  48 registers: five warps of
-// these buffers per SM quarter and more (40 registers spill: 330 us, 63
-// registers 309 us, without the loads ahead 314 us).
-// A warp with a row of more than kRowCols columns, or a mesh without room for
-// the chunks, takes its rows one after another, an incidence at a time.
+// each over the random columns of three rows.  48 registers: ten warps on each
+// quarter of an SM (40 registers spill: 330 us, 63 registers 309 us, without
+// the loads ahead 314 us).
+//
+// A mesh without room for the chunks, and a warp with a row of more than
+// kRowCols columns, read the incidences as they are, four at a time, in a loop
+// of their own (within the first it made that spill: 61^3 cube 329 us); such a
+// warp takes the rows that its buffers hold at 256 columns each (two of three,
+// three of five), then the others.  Buffers of 256 columns for every row cost
+// triangles 8 to 28% (900^2 square 225 -> 244 us, numbered at random 255 ->
+// 326: less room for L1).  40^3 cube of tets that share nothing: 685 us an
+// incidence at a time, 293 us four at a time; 10000 fans of 60 triangles 218
+// and 138 us.
 constexpr int kRowWarps = 4;
 constexpr int kRowCols = 160;
 constexpr int kRowStride = kRowCols + 11;  // the rows of a warp start 11 banks apart
-static_assert(3 * kRowStride >= kMaxCols, "one row of any length in the buffers of three");
+constexpr int kLongStride = 256;
+static_assert(kLongStride > kMaxCols && 3 * kRowStride >= kLongStride, "a row of any length in the buffers");
 
 template <int NB>
 __global__ void __launch_bounds__(kRowWarps * 32, 10)
     assemble_rows_kernel(const int32_t* __restrict__ inc_off, const int32_t* __restrict__ inc,
                          const uint8_t* __restrict__ colpos, const int32_t* __restrict__ row_ptr,
-                         const int32_t* __restrict__ choff, const int4* __restrict__ slot4,
-                         const uint32_t* __restrict__ pos4, int64_t chunk_cap, const float* __restrict__ A,
-                         const int32_t* n_rows_dev, float* __restrict__ val) {
+                         const int32_t* __restrict__ choff, const P2Plan* plan,
+                         const int32_t* __restrict__ col_idx, const float* __restrict__ A, float* __restrict__ val) {
   constexpr int G = 32 / NB;  // rows per warp
   constexpr int kWarpRows = G * kRowStride + 1;  // and a word for the lanes without a row
   __shared__ float acc_s[kRowWarps][kWarpRows];
@@ -1298,23 +1324,26 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
   for (int c = lane; c < kWarpRows; c += 32) rows[c] = 0.f;
   __syncwarp();
   const float* Aj = A + j;
-  int64_t r0 = (int64_t(blockIdx.x) * kRowWarps + warp) * G;
-  grid_wait(r0, n_rows_dev);
-  const int64_t n_rows = *n_rows_dev;
-  const bool chunked = choff[n_rows] <= chunk_cap;
-  const int64_t S = int64_t(gridDim.x) * kRowWarps * G;
+  int64_t first_row = (int64_t(blockIdx.x) * kRowWarps + warp) * G;
+  grid_wait(first_row, plan);
+  const uint32_t n_rows = plan->n_rows, S = gridDim.x * (kRowWarps * G);
+  // words from col_idx on to lane j's position in chunk 0, chunks being counted from col_idx too
+  const uint32_t chunk0 = plan->at, pos0 = 4 * (chunk0 + plan->n) - chunk0 * NB + j;
+  uint32_t r0 = uint32_t(first_row);
   if (r0 >= n_rows) return;  // warp-uniform: no CTA-wide barrier
   // chunks [c0, c0 + nch) of the lane's row, its first value, the values of the warp's rows
   struct Rows {
-    int32_t c0, nch, rp, total;
+    uint32_t c0;
+    int32_t nch, rp, total;
   };
-  auto load_rows = [&](int64_t q0) {
+  auto load_rows = [&](uint32_t q0) {
     Rows m{0, 0, 0, 0};
     if (q0 >= n_rows) return m;
-    const int64_t r = q0 + g;
+    const uint32_t r = q0 + g;
     const bool live = g < G && r < n_rows;
-    m.c0 = live ? __ldg(choff + r) : 0;
-    m.nch = live ? __ldg(choff + r + 1) - m.c0 : 0;
+    const int32_t c = live ? __ldg(choff + r) : 0;
+    m.c0 = chunk0 + c;
+    m.nch = live ? __ldg(choff + r + 1) - c : 0;
     m.rp = __ldg(row_ptr + (r < n_rows ? r : n_rows));
     m.total = __ldg(row_ptr + (q0 + G < n_rows ? q0 + G : n_rows));  // minus the first row's rp
     return m;
@@ -1325,14 +1354,16 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const bool on = k + h < m.nch;
-      const int64_t c = int64_t(m.c0) + k + h;
-      const int4 q = on ? __ldg(slot4 + c) : make_int4(-1, -1, -1, -1);
+      const uint32_t c = m.c0 + k + h;
+      const int4 q = on ? __ldg(reinterpret_cast<const int4*>(col_idx) + c) : make_int4(-1, -1, -1, -1);
       sn[4 * h] = q.x, sn[4 * h + 1] = q.y, sn[4 * h + 2] = q.z, sn[4 * h + 3] = q.w;
-      pn[h] = on ? __ldg(pos4 + c * NB + j) : 0u;
+      pn[h] = on ? __ldg(reinterpret_cast<const uint32_t*>(col_idx) + (pos0 + c * NB)) : 0u;  // below 2^32 words
     }
   };
+  bool left = !plan->fits;  // rows for the second loop
+  if (left) r0 = n_rows;
   Rows m = load_rows(r0);
-  if (chunked) load_chunks(m, 0);
+  load_chunks(m, 0);
   for (; r0 < n_rows; r0 += S) {
     const Rows mn = load_rows(r0 + S);
     const int32_t rp0 = __shfl_sync(0xffffffffu, m.rp, 0);
@@ -1340,7 +1371,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
 #pragma unroll
     for (int h = 0; h < G; ++h) first[h] = __shfl_sync(0xffffffffu, m.rp, h * NB) - rp0;
     first[G] = m.total - rp0;
-    bool fast = chunked;
+    bool fast = true;
 #pragma unroll
     for (int h = 0; h < G; ++h) fast &= first[h + 1] - first[h] <= kRowCols;
     if (fast) {
@@ -1378,31 +1409,63 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
       }
       __syncwarp();  // the row buffers are refilled for the next rows
     } else {
-      if (chunked) load_chunks(mn, 0);
-      for (int h = 0; h < G && r0 + h < n_rows; ++h) {
-        const int32_t tb = __ldg(inc_off + r0 + h), te = __ldg(inc_off + r0 + h + 1);
-        for (int32_t t = tb; t < te; ++t) {
-          if (lane < NB)
-            rows[__ldg(colpos + int64_t(t) * NB + lane)] += __ldg(A + int64_t(__ldg(inc + t)) * NB + lane);
-          __syncwarp();
-        }
-        const int32_t rp = __ldg(row_ptr + r0 + h), len = __ldg(row_ptr + r0 + h + 1) - rp;
-        for (int x = lane; x < len; x += 32) {
-          __stcs(val + int64_t(rp) + x, rows[x]);
-          rows[x] = 0.f;
-        }
-        __syncwarp();
-      }
+      left = true;
+      load_chunks(mn, 0);
     }
     m = mn;
+  }
+  if (!left) return;
+  // the rows passed over, without chunks; their bounds one group of rows ahead
+  struct Bounds {
+    int32_t rp, re, tb, te;
+  };
+  auto load_bounds = [&](uint32_t q0) {
+    const uint32_t r = q0 + g;
+    Bounds v{0, 0, 0, 0};
+    if (g < G && q0 < n_rows && r < n_rows)
+      v = {__ldg(row_ptr + r), __ldg(row_ptr + r + 1), __ldg(inc_off + r), __ldg(inc_off + r + 1)};
+    return v;
+  };
+  r0 = (blockIdx.x * kRowWarps + warp) * G;
+  for (Bounds v = load_bounds(r0), vn; r0 < n_rows; r0 += S, v = vn) {
+    vn = load_bounds(r0 + S);
+    const int len = v.re - v.rp;
+    const bool small = __all_sync(0xffffffffu, len <= kRowCols);
+    if (small && plan->fits) continue;
+    const int at_once = small ? G : kWarpRows / kLongStride, stride = small ? kRowStride : kLongStride;
+    for (int h0 = 0; h0 < G; h0 += at_once) {
+      const bool on = g >= h0 && g < h0 + at_once;
+      float* row = rows + (on ? (g - h0) * stride : 0);
+      const int n = on ? v.te - v.tb : 0;
+      const int steps = __reduce_max_sync(0xffffffffu, n);
+      for (int k0 = 0; k0 < steps; k0 += 4) {
+        int pos[4];
+        float a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = k0 + u < n;
+          pos[u] = in ? __ldg(colpos + int64_t(v.tb + k0 + u) * NB + j) : 0;
+          a[u] = in ? __ldg(Aj + int64_t(__ldg(inc + v.tb + k0 + u)) * NB) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (k0 + u < n) row[pos[u]] += a[u];
+          __syncwarp();
+        }
+      }
+      for (int c = j; c < (on ? len : 0); c += NB) {
+        __stcs(val + int64_t(v.rp) + c, row[c]);
+        row[c] = 0.f;
+      }
+      __syncwarp();  // the buffers are refilled for the next rows
+    }
   }
 }
 
 template <int NB>
 cudaError_t launch_p2_assemble(const AsmP2Layout& L, const float* A, float* val, cudaStream_t st) {
   return launch_chained(assemble_rows_kernel<NB>, grid_of(L.rows_cap, kRowWarps * (32 / NB)), kRowWarps * 32, 0, st,
-                        L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, L.choff, L.slot4, L.pos4, L.chunk_cap, A,
-                        L.n_rows, val);
+                        L.g2.inc_off, L.g2.inc, L.g2.colpos, L.g2.row_ptr, L.choff(), L.plan, L.g2.col_idx, A, val);
 }
 
 }  // namespace
@@ -1580,7 +1643,7 @@ fem_status fem_assembly_unknowns(const fem_mesh* mesh, int32_t form, const void*
   if (!ws || ws_bytes < P.bytes) return asm_fail(FEM_ERR_WORKSPACE, "assembly workspace too small");
   if (n_rows) {
     int32_t r = 0;
-    const cudaError_t e = cudaMemcpy(&r, P.n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost);
+    const cudaError_t e = cudaMemcpy(&r, &P.plan->n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) {
       fem::set_last_error("fem_assembly_unknowns: %s", cudaGetErrorString(e));
       return FEM_ERR_CUDA;
