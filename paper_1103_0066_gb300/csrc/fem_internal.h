@@ -192,7 +192,9 @@ cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned block, si
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess) cudaGetLastError();  // the status goes to the caller; its next call must not report it again
+  return e;
 }
 
 #ifdef __CUDACC__
