@@ -42,7 +42,7 @@ def form_info(form: int, dim: int):
     return nat.fem_form_info(form, dim)
 
 
-@functools.lru_cache(maxsize=None)
+@functools.lru_cache(maxsize=None, typed=True)  # 0.0 is not 0: ctypes refuses it
 def form_shape(form: int, dim: int):
     """(rows, cols) of the form's element blocks: (n, n), or (d+1, d * nbv) for
     the coupling forms DIV_P1P1 / DIV_P2P1."""
