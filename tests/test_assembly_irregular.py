@@ -12,7 +12,6 @@ import torch
 
 from paper_1103_0066_gb300 import meshgen as mg
 
-pytestmark = pytest.mark.gpu
 LP1, EP1 = 0, 2
 DEV = "cuda:0"
 RNG = np.random.default_rng
@@ -71,9 +70,44 @@ def _mesh(dim, shape):
     return _numbered(*_grid(dim, 11 if dim == 3 else 40), 6, elements=True)  # "shuffled"
 
 
+def _windows_by_count(conn, V, b):
+    """Which windows of short rows the build orders by incidence count (b: block size of the form)."""
+    nv = conn.shape[1]
+    slots = conn.ravel()
+    count = np.bincount(slots, minlength=V)
+    first = np.full(V, conn.size)
+    np.minimum.at(first, slots, np.arange(conn.size))
+    used = np.flatnonzero(count)
+    pairs = used[:-1][np.diff(used) == 1]
+    near = (np.abs(first[pairs + 1] - first[pairs]) <= 512).sum() * 2 >= len(pairs)
+    cols = np.bincount(np.unique(np.repeat(conn, nv, axis=1).ravel() * V + np.tile(conn, (1, nv)).ravel()) // V,
+                       minlength=V)
+    rows = used if near else used[np.argsort(first[used])]
+    rows = rows[(cols[rows] <= 32) & (count[rows] <= (32 if b == 1 else 255))]
+    size, blocks = {1: (32, 31), 2: (8, 127), 3: (3, 251)}[b]
+    out = []
+    for w in range(0, len(rows), size * blocks):
+        c = count[rows[w:w + size * blocks]]
+        c = np.pad(c, (0, -len(c) % size)).reshape(-1, size)
+        out.append(2 * size * c.max(1).sum() > 3 * c.sum())
+    return out
+
+
+SHAPES = ["edges", "unused", "windows", "split", "split random", "shuffled"]
+
+
 @pytest.mark.parametrize("dim", [2, 3])
 @pytest.mark.parametrize("form", [LP1, EP1])
-@pytest.mark.parametrize("shape", ["edges", "unused", "windows", "split", "split random", "shuffled"])
+def test_shapes_reach_both_orders(dim, form):
+    by_count = [_windows_by_count(*_mesh(dim, shape), dim if form == EP1 else 1) for shape in SHAPES]
+    assert any(any(w) for w in by_count) and any(not all(w) for w in by_count)
+    assert any(len(w) > 1 for w in by_count)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("form", [LP1, EP1])
+@pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("offset", [0, 1])
 def test_irregular_rows_bitwise(gfem, dim, form, shape, offset):
     conn, V = _mesh(dim, shape)
@@ -120,6 +154,7 @@ def _ns_per_incidence(gfem, conn, V, form, dim):
     return best / conn.numel()
 
 
+@pytest.mark.gpu
 @pytest.mark.parametrize("form,dim,shape", [(LP1, 3, "split"), (LP1, 3, "split random"), (LP1, 3, "half"),
                                             (LP1, 2, "split random"), (EP1, 3, "split random"), (EP1, 2, "eighth")])
 def test_irregular_mesh_costs_no_more_than_four_cubes(gfem, form, dim, shape):
