@@ -40,7 +40,7 @@ namespace {
 
 // CTA shape: one-warp CTAs on tets (no CTA-wide barrier), each holding the
 // four inverse Jacobians, their adjoints and sym(dA) in registers: 168 a
-// thread for P2 (104 bytes spilled), three warps on each quarter of an SM.
+// thread for P2 (100 bytes spilled), three warps on each quarter of an SM.
 template <int D, int FORM>
 struct IsoBwdShape {
   static constexpr int threads = D == 3 ? 32 : kTileElems;

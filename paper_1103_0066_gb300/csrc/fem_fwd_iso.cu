@@ -46,10 +46,10 @@ __device__ __forceinline__ void put_all(Sink& sink, const float* acc, std::integ
 
 // CTA shape: warps never wait for one another, so the CTA size only sets how
 // finely the register file is shared out.  On tets the P1 form runs one-warp
-// CTAs with at least 20 resident per SM, which holds it to 96 registers
-// without spills (21 warps per SM against 16 at 128 registers; 24 or 32 CTAs
-// spill and gain nothing); the P2 form with at least 16, which holds its 55
-// accumulators and four inverse Jacobians to 128 registers (20 bytes spilled).
+// CTAs with at least 20 resident per SM, which it reaches with 85 registers and
+// without spills (24 or 32 CTAs spill and gain nothing); the P2 form with at
+// least 16, which holds its 55 accumulators and four inverse Jacobians to 128
+// registers (28 bytes spilled).
 template <int D, int FORM>
 struct IsoShape {
   static constexpr bool tight = (D == 3);

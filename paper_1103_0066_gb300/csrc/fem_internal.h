@@ -174,11 +174,13 @@ cudaError_t ensure_smem(const void* kernel, size_t bytes);
 
 // Launch of a kernel that may be set up while the stream's previous kernel
 // ends (programmatic dependent launch): its CTAs take the places that the last
-// CTAs of that kernel leave, and grid_wait(), the kernel's first statement,
-// holds them until that kernel is complete and its writes are visible.  No
-// kernel here lets the next one begin earlier (launch_dependents): waiting
-// CTAs then took shared memory from running ones (128^3 cube, forward +
-// adjoint 478 -> 576 us, against 470 us without).
+// CTAs of that kernel leave, and grid_wait() holds them until that kernel is
+// complete and its writes are visible.  Every thread of a kernel launched this
+// way passes grid_wait() before its first access to global memory; indices and
+// shared memory may be set up before it.  No kernel here lets the next one
+// begin earlier (launch_dependents): waiting CTAs then took shared memory from
+// running ones (128^3 cube, forward + adjoint 478 -> 576 us, against 470 us
+// without).
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
                            const A&... args) {

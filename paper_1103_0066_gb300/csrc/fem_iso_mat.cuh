@@ -39,7 +39,7 @@ struct IsoMat {
 
 // p_{k,0} = -sum_{a>0} p_{k,a}; p_{k,a} = ji[k][a-1] for a > 0.
 template <int D>
-__host__ __device__ __forceinline__ void iso_p0(const float (&ji)[D + 1][D][D], float (&p0)[D + 1][D]) {
+__device__ __forceinline__ void iso_p0(const float (&ji)[D + 1][D][D], float (&p0)[D + 1][D]) {
 #pragma unroll
   for (int k = 0; k <= D; ++k)
 #pragma unroll
@@ -52,7 +52,7 @@ __host__ __device__ __forceinline__ void iso_p0(const float (&ji)[D + 1][D][D], 
 }
 
 template <int D>
-__host__ __device__ __forceinline__ float iso_dot(const float* u, const float* v) {
+__device__ __forceinline__ float iso_dot(const float* u, const float* v) {
   float s = u[0] * v[0];
 #pragma unroll
   for (int al = 1; al < D; ++al) s = fmaf(u[al], v[al], s);
@@ -64,7 +64,7 @@ __host__ __device__ __forceinline__ float iso_dot(const float* u, const float* v
 // the entries of index 0 from the zero row sums doubles the largest error
 // (8.0e-7 against 4.5e-7 of an element's largest entry, warped 128^3 cube).
 template <int D>
-__host__ __device__ __forceinline__ void iso_matrix_p1(const float (&ji)[D + 1][D][D], float* acc) {
+__device__ __forceinline__ void iso_matrix_p1(const float (&ji)[D + 1][D][D], float* acc) {
   constexpr int NV = D + 1;
   float p0[NV][D], P[NV][D];
   iso_p0<D>(ji, p0);
@@ -95,7 +95,7 @@ __host__ __device__ __forceinline__ void iso_matrix_p1(const float (&ji)[D + 1][
 
 // P2: acc[(i, j)] of the upper triangle, without the common factor.
 template <int D>
-__host__ __device__ __forceinline__ void iso_matrix_p2(const float (&ji)[D + 1][D][D], float* acc) {
+__device__ __forceinline__ void iso_matrix_p2(const float (&ji)[D + 1][D][D], float* acc) {
   using M = IsoMat<D>;
   constexpr int NV = M::NV;
   constexpr float n1 = M::n1, n2 = M::n2;
@@ -186,7 +186,7 @@ __host__ __device__ __forceinline__ void iso_matrix_p2(const float (&ji)[D + 1][
 // factor), p_{k,0} already folded in.  acc is homogeneous of degree two in p,
 // so sum_T s_T acc_T = sum u . p / 2 (Euler): the caller needs no acc.
 template <int D>
-__host__ __device__ __forceinline__ void iso_adjoint_p1(const float* s, const float (&ji)[D + 1][D][D],
+__device__ __forceinline__ void iso_adjoint_p1(const float* s, const float (&ji)[D + 1][D][D],
                                                         float (&u)[D + 1][D][D]) {
   constexpr int NV = D + 1;
   constexpr float n2 = IsoMat<D>::n2;
@@ -223,7 +223,7 @@ __host__ __device__ __forceinline__ void iso_adjoint_p1(const float* s, const fl
 }
 
 template <int D, class Sym>
-__host__ __device__ __forceinline__ void iso_adjoint_p2(const Sym& s, const float (&ji)[D + 1][D][D],
+__device__ __forceinline__ void iso_adjoint_p2(const Sym& s, const float (&ji)[D + 1][D][D],
                                                         float (&u)[D + 1][D][D]) {
   using M = IsoMat<D>;
   constexpr int NV = M::NV;
