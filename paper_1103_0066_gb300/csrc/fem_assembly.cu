@@ -240,8 +240,8 @@ __device__ __forceinline__ int row_kind(const int32_t* inc_off, const uint8_t* c
                                         int repeats, int64_t v) {
   const int len = row_ptr[v + 1] - row_ptr[v];
   const bool room = len <= BlockRows<B, ROW_SHORT>::cols;
-  if (B > 1) return room && !(repeats && row_repeats<NV>(inc_off, colpos, v)) ? ROW_SHORT : ROW_LONG;
-  if (len > BlockRows<B, ROW_WIDE>::cols) return ROW_LONG;
+  if constexpr (B > 1) return room && !(repeats && row_repeats<NV>(inc_off, colpos, v)) ? ROW_SHORT : ROW_LONG;
+  else if (len > BlockRows<B, ROW_WIDE>::cols) return ROW_LONG;
   return room && inc_off[v + 1] - inc_off[v] <= 32 ? ROW_SHORT : ROW_WIDE;
 }
 
@@ -617,10 +617,9 @@ __device__ __forceinline__ void assemble_block_rows(const BlockParams& p, const 
   auto load_slots = [&](const Head& h, int k0) {
     const int2* sl = p.slots + int64_t(h.s0) * K::unit + g;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const bool on = g < G && (k0 + u) * K::units < h.s1 - h.s0;
-      ahead[u] = on ? __ldg(sl + int64_t(k0 + u) * G) : make_int2(-1, int(kPad));
-    }
+    for (int u = 0; u < U; ++u)
+      ahead[u] = g < G && (k0 + u) * K::units < h.s1 - h.s0 ? __ldg(sl + int64_t(k0 + u) * G)
+                                                            : make_int2(-1, int(kPad));
   };
   int32_t rb = 0, re = 0;
   auto load_row = [&](const Head& h) {
