@@ -64,7 +64,7 @@ NCU_TRAFFIC = {
     "fem_bwd_elem_kernel<3,LAPLACE_P1,JAC_SAVED>": {"bytes_per_launch": 1315.6e6, "src": "f2c6ba2231620b53"},
     "fem_fwd_kernel<3,LAPLACE_P1,JAC_COMP>": {"bytes_per_launch": 961.6e6, "src": "21c79e41179ca40b"},
     "vertex_reduce_kernel<3>": {"bytes_per_launch": 149.2e6, "src": "fde8578fb91d3c94"},
-    "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 1433.4e6, "src": "2701c0cb95c89de5"},
+    "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 1433.6e6, "src": "b0bdc430e9be0a49"},
 }
 
 

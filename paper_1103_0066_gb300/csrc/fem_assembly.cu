@@ -1284,11 +1284,13 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
 // between lanes and a byte per incidence took two shuffles or loads for every
 // addition, on the pipe that the additions use (shared-memory and load pipe
 // 76% busy).  The next two chunks, of this row group or the next, are loaded
-// under the additions.  61^3 cube: 312 -> 277 us; bound by instruction issue
-// (68% active) and that pipe (70%), two accesses an addition, 2.6 wavefronts
+// under the additions.  61^3 cube: 312 -> 272 us; bound by instruction issue
+// (60% active) and that pipe (74%), two accesses an addition, 2.6 wavefronts
 // each over the random columns of three rows.  48 registers: ten warps on each
 // quarter of an SM (40 registers spill: 330 us, 63 registers 309 us, without
-// the loads ahead 314 us).
+// the loads ahead 314 us).  The rows' places in the output are formed after the
+// additions: held across them they spilled 8 bytes on triangles (900^2 square
+// 227 -> 218 us, numbered at random 262 -> 251).
 //
 // A mesh without room for the chunks, and a warp with a row of more than
 // kRowCols columns, read the incidences as they are, four at a time, in a loop
@@ -1297,8 +1299,8 @@ cudaError_t launch_p2_build(const int32_t* conn, int64_t n_elem, int64_t n_vert,
 // three of five), then the others.  Buffers of 256 columns for every row cost
 // triangles 8 to 28% (900^2 square 225 -> 244 us, numbered at random 255 ->
 // 326: less room for L1).  40^3 cube of tets that share nothing: 685 us an
-// incidence at a time, 293 us four at a time; 10000 fans of 60 triangles 218
-// and 138 us.
+// incidence at a time, 311 us four at a time; 10000 fans of 60 triangles 218
+// and 140 us.
 constexpr int kRowWarps = 4;
 constexpr int kRowCols = 160;
 constexpr int kRowStride = kRowCols + 11;  // the rows of a warp start 11 banks apart
@@ -1365,15 +1367,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
   load_chunks(m, 0);
   for (; r0 < n_rows; r0 += S) {
     const Rows mn = load_rows(r0 + S);
-    const int32_t rp0 = __shfl_sync(0xffffffffu, m.rp, 0);
-    int32_t first[G + 1];  // of each row, within the warp's run of values
-#pragma unroll
-    for (int h = 0; h < G; ++h) first[h] = __shfl_sync(0xffffffffu, m.rp, h * NB) - rp0;
-    first[G] = m.total - rp0;
-    bool fast = true;
-#pragma unroll
-    for (int h = 0; h < G; ++h) fast &= first[h + 1] - first[h] <= kRowCols;
-    if (fast) {
+    const int32_t end = __shfl_down_sync(0xffffffffu, m.rp, NB);  // of the lane's row
+    if (__all_sync(0xffffffffu, g >= G || (g < G - 1 ? end : m.total) - m.rp <= kRowCols)) {
       const int steps = __reduce_max_sync(0xffffffffu, m.nch);
       if (steps == 0) load_chunks(mn, 0);
       // two chunks at a time: their eight element rows, the next two chunks'
@@ -1398,7 +1393,11 @@ __global__ void __launch_bounds__(kRowWarps * 32, 10)
           }
         }
       }
-      for (int x = lane; x < first[G]; x += 32) {
+      const int32_t rp0 = __shfl_sync(0xffffffffu, m.rp, 0), total = m.total - rp0;
+      int32_t first[G];  // of each row, within the warp's run of values
+#pragma unroll
+      for (int h = 1; h < G; ++h) first[h] = __shfl_sync(0xffffffffu, m.rp, h * NB) - rp0;
+      for (int x = lane; x < total; x += 32) {
         int at = x;
 #pragma unroll
         for (int h = 1; h < G; ++h)
