@@ -471,7 +471,11 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
   }
   using SH = FwdShape<D, FORM, JAC, CT, OT>;
   const size_t per_warp = tma ? PL::tma_per_warp : PL::BULK ? PL::bulk_per_warp : PL::per_warp;
-  const int want = L.warps > 0 ? L.warps : SH::default_warps;
+  // CTAs per SM that a caller (or a kept choice of the autotuner) gives without
+  // the warps are CTAs of four, as on the other forms: of one, two CTAs per SM
+  // took 132 us on 900^2 x 2 P2 triangles, of four 56
+  const int own_warps = SH::rows36_100 && L.ctas_per_sm > 0 ? 4 : SH::default_warps;
+  const int want = L.warps > 0 ? L.warps : own_warps;
   const int warps = clamp_warps(want < SH::threads / 32 ? want : SH::threads / 32, per_warp);
   const size_t smem = size_t(warps) * per_warp + (tma ? 1024 : 0);
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
