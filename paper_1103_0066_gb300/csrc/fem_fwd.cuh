@@ -78,9 +78,16 @@ struct FwdShape {
 
 // How a warp stores its tile: through a padded stage and 16-byte stores
 // (ST_PLAIN: FP64 matrices, and the fused batch kernels, whose stage the
-// adjoint's dA shares), by one TMA tensor store (ST_TENSOR: 4 x 4 FP32) or by
-// a bulk copy of the stage (ST_BULK: 36 and 100 floats).
-enum : int { ST_PLAIN = 0, ST_TENSOR = 1, ST_BULK = 2 };
+// adjoint's dA shares), by one TMA tensor store (ST_TENSOR: 4 x 4 FP32), by a
+// bulk copy of the stage (ST_BULK: 36 and 100 floats) or, where A is not on a
+// 16-byte boundary, through the padded stage float by float (ST_SCALAR: 36, 100
+// and 144 floats).  As a branch beside the wide stores that loop has to stay
+// rolled (unrolled it costs them registers: P2 with a P1 coefficient 28.1 ->
+// 29.5 us at 40^3), which the unaligned call paid for: 40^3 cube, P2 36.7 us,
+// elasticity 54.8, P2 with a P1 coefficient 42.8; with kernels of its own 28.7,
+// 41.9 and 32.5.  FP64 matrices have no wide store beside it and unroll it too
+// (40^3 cube, P2 187.6 -> 170.1 us, elasticity 417 -> 382).
+enum : int { ST_PLAIN = 0, ST_TENSOR = 1, ST_BULK = 2, ST_SCALAR = 3 };
 
 // Shared-memory plan of one warp.
 template <int D, int FORM, class CT, class OT>
@@ -101,6 +108,7 @@ struct FwdPlan {
   static constexpr bool BULK = sizeof(OT) == 4 && NN % 4 == 0 && (NN / 4) % 2 == 1;
   static constexpr size_t bulk_per_warp = size_t(32) * NN * sizeof(OT);
   static constexpr int plain_store = BULK ? ST_BULK : ST_PLAIN;  // without a tensor map
+  static constexpr bool SCALAR = sizeof(OT) == 4 && NN % 4 == 0 && !SWZ16;  // has an ST_SCALAR kernel
   static constexpr size_t stage_of(int st) {
     return st == ST_TENSOR ? tma_per_warp : st == ST_BULK ? bulk_per_warp : per_warp;
   }
@@ -281,7 +289,9 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
     fill(sink);
     __syncwarp();
     bool done = false;
-    if constexpr (SST == NN) {  // unpadded rows of odd size: the stage is the tile as it lies in memory
+    constexpr bool wide = ST != ST_SCALAR && (SST == NN || (sizeof(OT) == 4 && NN % 4 == 0));
+    if constexpr (!wide) {
+    } else if constexpr (SST == NN) {  // unpadded rows of odd size: the stage is the tile as it lies in memory
       constexpr int W = 16 / sizeof(OT);
       if (p.vec_store) {
         const int nq = cnt * NN / W;
@@ -292,7 +302,7 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
         for (int idx = W * nq + lane; idx < cnt * NN; idx += 32) __stcs(dst + idx, st[idx]);
         done = true;
       }
-    } else if constexpr (sizeof(OT) == 4 && NN % 4 == 0) {
+    } else {
       if (p.vec_store) {
         const int nq = cnt * (NN / 4);
         for (int q = lane; q < nq; q += 32) {
@@ -306,7 +316,7 @@ __device__ __forceinline__ void fwd_fill_store(const FwdParams<CT, OT>& p, int64
     }
     if (!done) {
       const int nw = cnt * NN;
-#pragma unroll 1
+#pragma unroll (wide ? 1 : 4)
       for (int idx = lane; idx < nw; idx += 32) {
         const int el = idx / NN;
         __stcs(dst + idx, st[el * SST + (idx - el * NN)]);
@@ -441,7 +451,7 @@ __global__ void __launch_bounds__(FwdShape<D, FORM, JAC, CT, OT>::threads, FwdSh
     fwd_step<D, FORM, JAC, CT, OT, ST>(p, t, S, lane, vb, va, Xb, Xa, fb, wb, fa, wa, st2, &tmap, err);
     if ((t += S) >= ntiles) break;
   }
-  if constexpr (ST != ST_PLAIN) bulk_wait<0>();  // the stages outlive every copy that reads them
+  if constexpr (TMA || ST == ST_BULK) bulk_wait<0>();  // the stages outlive every copy that reads them
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && p.dev_err) atomicOr(p.dev_err, err);
 }
@@ -470,17 +480,24 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
     }
   }
   using SH = FwdShape<D, FORM, JAC, CT, OT>;
-  const size_t per_warp = tma ? PL::tma_per_warp : PL::BULK ? PL::bulk_per_warp : PL::per_warp;
+  bool scalar = false;
+  if constexpr (PL::SCALAR) {
+    if (!p.vec_store) {
+      scalar = true;
+      kern = fem_fwd_kernel<D, FORM, JAC, CT, OT, ST_SCALAR>;
+    }
+  }
+  const size_t per_warp = PL::stage_of(tma ? ST_TENSOR : scalar ? ST_SCALAR : PL::plain_store);
   // CTAs per SM that a caller (or a kept choice of the autotuner) gives without
   // the warps are CTAs of four, as on the other forms: of one, two CTAs per SM
   // took 132 us on 900^2 x 2 P2 triangles, of four 56
-  const int own_warps = SH::rows36_100 && L.ctas_per_sm > 0 ? 4 : SH::default_warps;
+  const int own_warps = SH::rows36_100 && (scalar || L.ctas_per_sm > 0) ? 4 : SH::default_warps;
   const int want = L.warps > 0 ? L.warps : own_warps;
   const int warps = clamp_warps(want < SH::threads / 32 ? want : SH::threads / 32, per_warp);
   const size_t smem = size_t(warps) * per_warp + (tma ? 1024 : 0);
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
-  const int ctas = L.ctas_per_sm > 0 || L.warps > 0 ? L.ctas_per_sm : SH::default_ctas;
+  const int ctas = L.ctas_per_sm > 0 || L.warps > 0 || scalar ? L.ctas_per_sm : SH::default_ctas;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, ctas);
   return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p, tmap);
 }
