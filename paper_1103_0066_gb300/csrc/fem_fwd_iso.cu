@@ -62,16 +62,16 @@ struct IsoShape {
 // beside the 12.8 KB output stage cost more resident warps than the wait saved
 // (64^3 cube, forward + adjoint 386 against 381 us; P1 tets 173 -> 168 us, P2
 // triangles at 700 x 700 x 2 111 -> 100 us).
-template <int D, int FORM>
+template <int D, int FORM, int ST>
 struct IsoFwdPlan {
   using PL = FwdPlan<D, FORM, float, float>;
   static constexpr bool ahead = D == 2 || FORM == LAPLACE_P1_ISO;
-  static constexpr size_t stage = PL::stage_of(PL::plain_store);
+  static constexpr size_t stage = PL::stage_of(ST);
   static constexpr size_t mid_bytes = align_up(size_t(32) * (D * D * (D + 1) / 2) * 4, 128);
   static constexpr size_t per_warp = stage + (ahead ? mid_bytes + 32 * (D + 1) * D * 4 : 0);
 };
 
-template <int D, int FORM>
+template <int D, int FORM, int ST>
 __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>::min_ctas)
     fem_fwd_iso_kernel(FwdParams<float, float> p, const float* __restrict__ mid) {
   using FT = FormTraits<D, FORM>;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
   constexpr int NE = D * (D + 1) / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  using IP = IsoFwdPlan<D, FORM>;
+  using IP = IsoFwdPlan<D, FORM, ST>;
   unsigned char* wbase = smem_raw + size_t(warp) * IP::per_warp;
   float* st = reinterpret_cast<float*>(wbase);
   float* ms = reinterpret_cast<float*>(wbase + IP::stage);                         // [32][NE * D]
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
     } else {
       load_conn<D>(p.conn, e + S * 32, p.n_elem, p.vec_conn, v);
     }
-    fwd_fill_store<D, FORM, float, float, PL::plain_store>(
+    fwd_fill_store<D, FORM, float, float, ST>(
         p, t, lane,
         [&](auto& sink) {
           float acc[FT::NT];
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(IsoShape<D, FORM>::threads, IsoShape<D, FORM>:
         st, nullptr);
   }
   cp_async_wait<0>();
-  if constexpr (PL::BULK) bulk_wait<0>();  // the stage outlives every copy that reads it
+  if constexpr (ST == ST_BULK) bulk_wait<0>();  // the stage outlives every copy that reads it
   err = __reduce_or_sync(0xffffffffu, err);
   if (err && lane == 0 && p.dev_err) atomicOr(p.dev_err, err);
 }
@@ -175,9 +175,14 @@ cudaError_t launch_iso_t(const FwdLaunch& L, const float* mid) {
   p.dev_err = L.dev_err;
   p.vec_conn = (D == 3) && (reinterpret_cast<uintptr_t>(L.conn) % 16 == 0);
   p.vec_store = (reinterpret_cast<uintptr_t>(L.A) % 16 == 0);
-  auto kern = fem_fwd_iso_kernel<D, FORM>;
+  using PL = FwdPlan<D, FORM, float, float>;
+  constexpr int unaligned = PL::SCALAR ? ST_SCALAR : PL::plain_store;
+  const bool wide = p.vec_store || !PL::SCALAR;
+  auto kern = wide ? fem_fwd_iso_kernel<D, FORM, PL::plain_store> : fem_fwd_iso_kernel<D, FORM, unaligned>;
   const int warps = IsoShape<D, FORM>::threads / 32;
-  const size_t smem = size_t(warps) * IsoFwdPlan<D, FORM>::per_warp;
+  const size_t per_warp =
+      wide ? IsoFwdPlan<D, FORM, PL::plain_store>::per_warp : IsoFwdPlan<D, FORM, unaligned>::per_warp;
+  const size_t smem = size_t(warps) * per_warp;
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, L.ctas_per_sm);
