@@ -65,7 +65,8 @@ struct FwdShape {
   static constexpr int threads = tight ? 32 : 512;
   static constexpr int min_ctas = tight ? tight_ctas() : 1;
   // 36 and 100 floats a row (stored by bulk copies): one-warp CTAs
-  static constexpr bool rows36_100 = sizeof(OT) == 4 && (FormTraits<D, FORM>::NN == 36 || FormTraits<D, FORM>::NN == 100);
+  static constexpr bool rows36_100 =
+      sizeof(OT) == 4 && (FormTraits<D, FORM>::NN == 36 || FormTraits<D, FORM>::NN == 100);
   static constexpr int default_warps = tight || rows36_100 ? 1 : 4;
   // CTAs per SM of the default grid, 0 for as many as are resident.  More than
   // that lets the hardware hand the last tiles to whichever SM is free, which
@@ -73,7 +74,9 @@ struct FwdShape {
   // coefficient 72^3 159 -> 151, 36-float rows at 1023 x 1023 x 2 59.5 -> 56,
   // elasticity 61^3 140 -> 137.  The 3D P1 forward, bound by latency, and the
   // adjoints, whose warps start with an exposed copy, lose by it.
-  static constexpr int default_ctas = rows36_100 ? 64 : (D == 3 && FORM == ELASTIC_P1 && sizeof(OT) == 4) ? 8 : 0;
+  // FP64 coordinates take more registers and lose by it (elasticity 56^3 614 -> 634).
+  static constexpr int default_ctas =
+      rows36_100 ? 64 : (D == 3 && FORM == ELASTIC_P1 && sizeof(OT) == 4 && sizeof(CT) == 4) ? 8 : 0;
 };
 
 // How a warp stores its tile: through a padded stage and 16-byte stores
@@ -497,7 +500,14 @@ cudaError_t launch_fwd_t(const FwdLaunch& L) {
   const size_t smem = size_t(warps) * per_warp + (tma ? 1024 : 0);
   cudaError_t st = ensure_smem(reinterpret_cast<const void*>(kern), smem);
   if (st != cudaSuccess) return st;
-  const int ctas = L.ctas_per_sm > 0 || L.warps > 0 || scalar ? L.ctas_per_sm : SH::default_ctas;
+  // A caller's warps alone, and an unaligned output, keep to the resident CTAs
+  // except on many tiles, where the wider grid pays for any number of warps
+  // (36-float rows at 1400 x 1400 x 2: 108 -> 101 us; at 500 x 500 x 2, 14 -> 16)
+  const bool many = SH::rows36_100 && (L.n_elem + 31) / 32 >= int64_t(8) * 64 * device_sm_count();
+  const int ctas = L.ctas_per_sm > 0                ? L.ctas_per_sm
+                   : L.warps <= 0 && !scalar        ? SH::default_ctas
+                   : many && 64 / warps > 0         ? 64 / warps
+                                                    : 0;
   const unsigned grid = pipeline_grid(reinterpret_cast<const void*>(kern), warps, smem, L.n_elem, ctas);
   return launch_chained(kern, grid, unsigned(warps * 32), smem, L.stream, p, tmap);
 }
