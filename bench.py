@@ -61,9 +61,9 @@ KERNEL_SOURCES = {
 # forward's and the reduction's scaled figures are lower bounds: the part of
 # their output still dirty in L2 when the kernel ends does not grow with it.
 NCU_TRAFFIC = {
-    "fem_bwd_elem_kernel<3,LAPLACE_P1,JAC_SAVED>": {"bytes_per_launch": 1315.9e6, "src": "8d0498a3d8618799"},
-    "fem_fwd_kernel<3,LAPLACE_P1,JAC_COMP>": {"bytes_per_launch": 962.0e6, "src": "6a1402a65ee08657"},
-    "vertex_reduce_kernel<3>": {"bytes_per_launch": 149.2e6, "src": "fde8578fb91d3c94"},
+    "fem_bwd_elem_kernel<3,LAPLACE_P1,JAC_SAVED>": {"bytes_per_launch": 1316.4e6, "src": "1283e71157bf367b"},
+    "fem_fwd_kernel<3,LAPLACE_P1,JAC_COMP>": {"bytes_per_launch": 962.4e6, "src": "917d0c43ea376463"},
+    "vertex_reduce_kernel<3>": {"bytes_per_launch": 149.3e6, "src": "fde8578fb91d3c94"},
     "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 1433.6e6, "src": "b0bdc430e9be0a49"},
 }
 

@@ -74,7 +74,7 @@ struct FwdShape {
   // coefficient 72^3 159 -> 151, 36-float rows at 1023 x 1023 x 2 59.5 -> 56,
   // elasticity 61^3 140 -> 137.  The 3D P1 forward, bound by latency, and the
   // adjoints, whose warps start with an exposed copy, lose by it.
-  // FP64 coordinates take more registers and lose by it (elasticity 56^3 614 -> 634).
+  // FP64 coordinates take more registers and lose by it (elasticity 72^3 614 -> 634).
   static constexpr int default_ctas =
       rows36_100 ? 64 : (D == 3 && FORM == ELASTIC_P1 && sizeof(OT) == 4 && sizeof(CT) == 4) ? 8 : 0;
 };
