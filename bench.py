@@ -64,7 +64,7 @@ NCU_TRAFFIC = {
     "fem_bwd_elem_kernel<3,LAPLACE_P1,JAC_SAVED>": {"bytes_per_launch": 1316.4e6, "src": "1283e71157bf367b"},
     "fem_fwd_kernel<3,LAPLACE_P1,JAC_COMP>": {"bytes_per_launch": 962.4e6, "src": "917d0c43ea376463"},
     "vertex_reduce_kernel<3>": {"bytes_per_launch": 149.3e6, "src": "fde8578fb91d3c94"},
-    "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 1433.6e6, "src": "b0bdc430e9be0a49"},
+    "fem_assemble<LAPLACE_P1>": {"bytes_per_launch": 1433.1e6, "src": "736ebac3d8eab17e"},
 }
 
 

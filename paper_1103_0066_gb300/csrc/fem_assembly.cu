@@ -781,8 +781,8 @@ __device__ __forceinline__ void assemble_block_rows(const BlockParams& p, const 
 // of A, 8 bytes per incidence and the values (108 bytes per tet of a scalar
 // form, against 197 with records), and because a lane's sums need neither
 // atomics nor barriers.  Scalar forms, 96^3 cube: 241 us (tile pass 190 and
-// entry pass 48) -> 134 us; elasticity, 56^3 cube: 517 us (a thread per row,
-// 5.5 warps per SM) -> 149 us, 4.8 TB/s of the bytes it cannot do without.
+// entry pass 48) -> 124 us; elasticity, 56^3 cube: 517 us (a thread per row,
+// 5.5 warps per SM) -> 146 us, 4.9 TB/s of the bytes it cannot do without.
 // What bounds it: the L1 and shared-memory pipe (two or three conflict-free
 // accesses a contribution, and a tag look-up per element row).
 // The long rows come first, then the wide ones: they take longest.

@@ -59,7 +59,7 @@ def test_each_form_sees_its_own_inputs(gfem, how, dim, form):
     cm, mid0 = mg.curved_mesh(m)
     form = getattr(gfem, form)
     conn = torch.from_numpy(m.conn).to(DEV)
-    base, mid = torch.from_numpy(cm.coords.astype(np.float32)).to(DEV), torch.from_numpy(mid0.astype(np.float32)).to(DEV)
+    base, mid = (torch.from_numpy(t.astype(np.float32)).to(DEV) for t in (cm.coords, mid0))
     V, E = base.shape[0], conn.shape[0]
     c0 = 1 + torch.rand(V if w1 else E, generator=torch.Generator(DEV).manual_seed(1), device=DEV)
     x, md, c = base.clone(), mid.clone(), c0.clone()

@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dim,form", [(2, "LAPLACE_P2"), (2, "ELASTIC_P1"), (3, "LAPLACE_P2_W1")])
 def test_ctas_per_sm_alone(gfem, dim, form):
     form = getattr(gfem, form)
-    m = mg.square_tri_mesh(700, 0.2, mg.rng_for(1), np.float32) if dim == 2 else mg.cube_tet_mesh(48, 0.15, mg.rng_for(1))
+    m = (mg.square_tri_mesh(700, 0.2, mg.rng_for(1), np.float32) if dim == 2 else
+         mg.cube_tet_mesh(48, 0.15, mg.rng_for(1)))
     x, conn = torch.from_numpy(m.coords).cuda(), torch.from_numpy(m.conn).cuda()
     w = torch.ones(m.n_vert, device="cuda") if form == gfem.LAPLACE_P2_W1 else None
     A, B = (torch.empty((m.n_elem,) + gfem.form_shape(form, dim), device="cuda") for _ in range(2))

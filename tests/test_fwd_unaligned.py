@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dim,form", [(2, "LAPLACE_P2_W1"), (3, "LAPLACE_P2"), (3, "ELASTIC_P1")])
 def test_unaligned_output_time(gfem, dim, form):
     form = getattr(gfem, form)
-    m = mg.square_tri_mesh(500, 0.2, mg.rng_for(1), np.float32) if dim == 2 else mg.cube_tet_mesh(40, 0.15, mg.rng_for(1))
+    m = (mg.square_tri_mesh(500, 0.2, mg.rng_for(1), np.float32) if dim == 2 else
+         mg.cube_tet_mesh(40, 0.15, mg.rng_for(1)))
     x, conn = torch.from_numpy(m.coords).cuda(), torch.from_numpy(m.conn).cuda()
     w = torch.ones(m.n_vert, device="cuda") if form == gfem.LAPLACE_P2_W1 else None
     shape = (m.n_elem,) + gfem.form_shape(form, dim)
@@ -41,7 +42,8 @@ def test_unaligned_output_time(gfem, dim, form):
 @pytest.mark.parametrize("dim", [2, 3])
 def test_unaligned_curved_output_time(gfem, dim):
     """Curved P2: 1.36 and 1.44 times the aligned call with the rolled loop."""
-    m = mg.square_tri_mesh(1000, 0.2, mg.rng_for(1), np.float32) if dim == 2 else mg.cube_tet_mesh(56, 0.15, mg.rng_for(1))
+    m = (mg.square_tri_mesh(1000, 0.2, mg.rng_for(1), np.float32) if dim == 2 else
+         mg.cube_tet_mesh(56, 0.15, mg.rng_for(1)))
     cm, mid = mg.curved_mesh(m)
     x, conn, mid = (torch.from_numpy(t).cuda() for t in (cm.coords.astype(np.float32), m.conn, mid))
     shape = (m.n_elem,) + gfem.form_shape(gfem.LAPLACE_P2_ISO, dim)
